@@ -192,6 +192,15 @@ __device__ __forceinline__ T band_a(const T* kx, const T* ky, int n0, int r, int
     return T(0);
 }
 
+// Diagonal of row j of h0^2 A_0: the sum of the cell's four faces.
+template <typename T>
+__device__ __forceinline__ double level0_diag(const T* kx, const T* ky, int n0, int j)
+{
+    const int j1 = j % n0, j2 = j / n0;
+    return widen(kx[j2 * kx_pitch(n0) + j1]) + widen(kx[j2 * kx_pitch(n0) + j1 + 1]) + widen(ky[j2 * n0 + j1]) +
+           widen(ky[(j2 + 1) * n0 + j1]);
+}
+
 // Factor, exact FP64 solve with f = 1, F_0; the mixed forms also keep an FP32
 // copy of the factor for the coarse solves of their FP32 V-cycles.
 template <typename T, bool MX>
@@ -289,6 +298,19 @@ __global__ void kb_coarse(FmgArgs A, int B)
     }
 }
 
+// F_0 of a level-0 solution x(r), r < N: the mean from sixteen partial sums
+// (x of r = c mod 16 in ascending r) added pairwise, or the mean of the four
+// centre cells. One order for the kernels that run a sample on one thread and
+// on several lanes.
+__device__ __forceinline__ double tree16(double (&s)[16])
+{
+#pragma unroll
+    for (int w = 8; w > 0; w >>= 1)
+#pragma unroll
+        for (int c = 0; c < w; ++c) s[c] += s[c + w];
+    return s[0];
+}
+
 // Level 0 for n0 = NC fixed at compile time, one thread per sample, with the
 // working rows of the factorisation in shared memory: column j of L needs
 // rows j..j+NC only, so a ring of NC+1 rows per thread (transposed by thread:
@@ -297,8 +319,8 @@ __global__ void kb_coarse(FmgArgs A, int B)
 // values in registers and every value stored into the sample's solution
 // array, which the backward substitution then overwrites in place (again
 // with the last NC values in registers); shared memory holds the ring only,
-// so that all samples of a call fit on the GPU at once. Same arithmetic, in
-// the same order, as kb_level0.
+// so that all samples of a call fit on the GPU at once. Every sum takes its
+// oldest term first, the order in which kb_level0_lanes' updates arrive.
 template <typename T, bool MX, int NC>
 __global__ void __launch_bounds__(64) kb_level0_fixed(FmgArgs A, int B)
 {
@@ -326,23 +348,17 @@ __global__ void __launch_bounds__(64) kb_level0_fixed(FmgArgs A, int B)
             constexpr bool FULL = decltype(full)::value;
             const int s0 = j % W;
             auto slot = [&](int l) { return s0 + l >= W ? s0 + l - W : s0 + l; };  // slot of row j + l
-            const int j1 = j % NC, j2 = j / NC;
-            double d = widen(L0.kx[j2 * kx_pitch(NC) + j1]) + widen(L0.kx[j2 * kx_pitch(NC) + j1 + 1]) +
-                       widen(L0.ky[j2 * NC + j1]) + widen(L0.ky[(j2 + 1) * NC + j1]);
+            double d = level0_diag(L0.kx, L0.ky, NC, j);
+            double v = h2;  // forward substitution, f = 1
 #pragma unroll
-            for (int q = 1; q <= NC; ++q) {
-                if (!FULL && q > j) break;
+            for (int q = NC; q >= 1; --q) {
+                if (!FULL && q > j) continue;
                 const double l = Rs(s0, q);
-                d -= l * l;
+                d = fma(-l, l, d);
+                v = fma(-l, win[q - 1], v);
             }
             const double rl = rsqrt64(d);
             Rs(s0, 0) = rl;
-            double v = h2;  // forward substitution, f = 1
-#pragma unroll
-            for (int q = 1; q <= NC; ++q) {
-                if (!FULL && q > j) break;
-                v -= Rs(s0, q) * win[q - 1];
-            }
             const double yj = v * rl;
             x[j] = yj;
 #pragma unroll
@@ -363,10 +379,10 @@ __global__ void __launch_bounds__(64) kb_level0_fixed(FmgArgs A, int B)
                 if constexpr (FULL) {
 #pragma unroll
                     for (int u = 0; u < NC - l; ++u) {  // tt = r - NC + u = j - (NC - l) + u
-                        a -= Rs(sr, NC - u) * Rs(s0, NC - l - u);
+                        a = fma(-Rs(sr, NC - u), Rs(s0, NC - l - u), a);
                     }
                 } else {
-                    for (int tt = (r - NC > 0 ? r - NC : 0); tt < j; ++tt) a -= Rs(sr, r - tt) * Rs(s0, j - tt);
+                    for (int tt = (r - NC > 0 ? r - NC : 0); tt < j; ++tt) a = fma(-Rs(sr, r - tt), Rs(s0, j - tt), a);
                 }
                 Rs(sr, l) = a * rl;
             }
@@ -379,8 +395,8 @@ __global__ void __launch_bounds__(64) kb_level0_fixed(FmgArgs A, int B)
         for (int r = N - 1; r >= 0; --r) {
             double v = x[r];
 #pragma unroll
-            for (int q = 1; q <= NC; ++q)
-                if (r + q < N) v -= fac[static_cast<size_t>((r + q) * W + q) * cs + i] * win[q - 1];
+            for (int q = NC; q >= 1; --q)
+                if (r + q < N) v = fma(-fac[static_cast<size_t>((r + q) * W + q) * cs + i], win[q - 1], v);
             const double xr = v * fac[static_cast<size_t>(r * W) * cs + i];
             x[r] = xr;
 #pragma unroll
@@ -390,9 +406,14 @@ __global__ void __launch_bounds__(64) kb_level0_fixed(FmgArgs A, int B)
         }
         double F0;
         if (A.qoi == MLQMC_QOI_MEAN) {
-            double acc = 0.0;
-            for (int r = 0; r < N; ++r) acc += x[r];
-            F0 = acc / static_cast<double>(N);
+            double acc[16];
+#pragma unroll
+            for (int c = 0; c < 16; ++c) acc[c] = x[c];
+            for (int r = 16; r < N; r += 16)
+#pragma unroll
+                for (int c = 0; c < 16; ++c)
+                    if (N % 16 == 0 || r + c < N) acc[c] += x[r + c];
+            F0 = tree16(acc) / static_cast<double>(N);
         } else {
             constexpr int m = NC / 2;
             F0 = 0.25 * (x[(m - 1) * NC + (m - 1)] + x[(m - 1) * NC + m] + x[m * NC + (m - 1)] + x[m * NC + m]);
@@ -401,144 +422,191 @@ __global__ void __launch_bounds__(64) kb_level0_fixed(FmgArgs A, int B)
     }
 }
 
-// Level 0 for n0 = NC for calls of few samples: the same factorisation,
-// substitutions and F_0 as kb_level0_fixed, every operation in its order, but
-// each step of the factorisation split over the NC + 2 warps of a CTA that
-// holds 32 samples (lane = sample). On GB300 an FP64 warp instruction holds
-// its SM sub-partition for about 70 cycles whatever its active lanes, so one
-// thread's ~4,700 FP64 operations take 0.15 ms or more however few samples a
-// call has. Split this way a step's FP64 work runs on several sub-partitions
-// at once; what remains per step is the dependent chain of the reciprocal
-// square root and the shared FP64 pipes (about 0.18 ms per call). Step j:
-// warp 0 forms d_j and 1/L(j,j) (the face sum of d_j formed one step ahead by
-// warp NC, whose band row is the shortest), warp l (1..NC) the dot product of
-// row j+l, warp NC+1 the forward value; after a barrier warp l scales its entry of
-// column j, warp NC+1 finishes y_j and warp 0 writes the finished row j to
-// the global factor; a second barrier ends the step. Warp NC+1 then runs the
-// backward substitution (the factor rows from global memory, written by warp
-// 0 before the barriers) and forms F_0. The ring of NC+1 rows and the
-// forward values of the group's samples sit in shared memory. Lanes past B
-// compute on sample B-1 and store nothing.
-template <typename T, bool MX, int NC>
-__global__ void __launch_bounds__(32 * (NC + 2)) kb_level0_split(FmgArgs A, int B)
+// Level 0 for n0 = NC on several lanes per sample (LPR lanes for each of the
+// NC rows of the working window, NC LPR lanes in all). On GB300 an FP64 warp
+// instruction holds its SM sub-partition for about 70 cycles whatever its
+// active lanes, so what a sample costs is its FP64 warp instructions, and one
+// thread's ~4,700 of them take 0.2 ms however few samples a call has. Here
+// column j updates the whole trailing window at once (right-looking): lane
+// (p, g) keeps row r = p mod NC and its columns c = g mod LPR in registers
+// (register c mod NC), the diagonal and the right-hand side ride along, and a
+// column costs its reciprocal square root (5), one scaling and NC/LPR + 1 (or
+// + 3, LPR = 1) updates. Registers whose column is already eliminated take
+// part with stale values and are reset when their row is replaced; the
+// finished column goes to shared memory (backward substitution, pushed the
+// same way) and to the global factor. Sums take their oldest term first, as
+// in kb_level0_fixed: the same bits.
+template <int NC, int LPR>
+struct L0Geom {
+    static constexpr int TL = NC * LPR;      // lanes that work on a sample
+    static constexpr int SEG = TL <= 4 ? 4 : (TL <= 8 ? 8 : (TL <= 16 ? 16 : 32));  // lanes that a sample occupies
+    static constexpr int SPW = 32 / SEG;     // samples per warp
+    static constexpr int N = NC * NC;
+    static constexpr int oL = 0;             // column j of L below the diagonal: [j * NC + row mod NC]
+    static constexpr int oR = oL + N * NC;   // 1 / L(j, j)
+    static constexpr int oY = oR + N;        // forward values, then the solution
+    static constexpr int oD = oY + N;        // diagonal sums of h0^2 A_0
+    static constexpr int oA = oD + N;        // -L.kx: coupling of row r to r - 1, then of row r to r - NC
+    static constexpr int per = oA + 2 * N;   // doubles per sample
+    static constexpr size_t bytes = sizeof(double) * per * SPW;
+};
+
+template <typename T, bool MX, int NC, int LPR>
+__global__ void __launch_bounds__(32) kb_level0_lanes(FmgArgs A, int B)
 {
-    constexpr int N = NC * NC, W = NC + 1;
-    __shared__ double ring[W * W * 32];  // [(slot * W + e) * 32 + lane]
-    __shared__ double ys[N * 32];        // forward values, then the solution
-    __shared__ double dg[2 * 32];        // the diagonal sum of the next step, formed one step ahead
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    using Gm = L0Geom<NC, LPR>;
+    constexpr int N = NC * NC, W = NC + 1, KR = (NC + LPR - 1) / LPR;
+    static_assert(LPR == 1 || LPR == 4, "the diagonal and the right-hand side take two groups, the column a third");
+    extern __shared__ double l0sh[];
+    const int lane = threadIdx.x, team = lane / Gm::SEG, tl = lane - team * Gm::SEG;
+    const int i = blockIdx.x * Gm::SPW + team;
+    const bool live = i < B;
+    const int si = live ? i : B - 1;  // lanes past B compute on sample B-1 and store nothing
+    const bool work = tl < Gm::TL;    // NC = 6: lanes past the window stay idle but converged
+    const int p = work ? tl / LPR : 0, g = work ? tl - p * LPR : 0;
+    const int t0 = team * Gm::SEG;
+    double* S = l0sh + static_cast<size_t>(team) * Gm::per;
     const size_t cs = A.chol.stride;
     double* fac = reinterpret_cast<double*>(A.chol.base);
     float* f32 = reinterpret_cast<float*>(A.chol32);
     const double h2 = 1.0 / (static_cast<double>(NC) * NC);
-    auto Rs = [&](int slot, int e) -> double& { return ring[(slot * W + e) * 32 + lane]; };
-    for (int base = blockIdx.x * 32; base < B; base += gridDim.x * 32) {
-        const int i = base + lane;
-        const bool live = i < B;
-        const int si = live ? i : B - 1;
-        const Lv<T> L0 = view<T>(A, 0, si);
-        double win[NC];  // forward substitution: win[q - 1] = y_(j - q)
-#pragma unroll
-        for (int q = 0; q < NC; ++q) win[q] = 0.0;
-        auto step = [&](int j, auto full) {
-            constexpr bool FULL = decltype(full)::value;
-            const int s0 = j % W;
-            double a = 0.0, v = 0.0;
-            int sr = 0;
-            const int l = warp;  // row j + l for warps 1..NC
-            // the face sum of row jj's diagonal, in kb_level0_fixed's order
-            auto diag_sum = [&](int jj) {
-                const int j1 = jj % NC, j2 = jj / NC;
-                return widen(L0.kx[j2 * kx_pitch(NC) + j1]) + widen(L0.kx[j2 * kx_pitch(NC) + j1 + 1]) +
-                       widen(L0.ky[j2 * NC + j1]) + widen(L0.ky[(j2 + 1) * NC + j1]);
-            };
-            if (warp == 0) {
-                double d = j == 0 ? diag_sum(0) : dg[(j & 1) * 32 + lane];  // step j > 0: formed by warp NC
-#pragma unroll
-                for (int q = 1; q <= NC; ++q) {
-                    if (!FULL && q > j) break;
-                    const double lq = Rs(s0, q);
-                    d -= lq * lq;
-                }
-                Rs(s0, 0) = rsqrt64(d);
-            } else if (warp <= NC) {
-                if (warp == NC && j + 1 < N) dg[((j + 1) & 1) * 32 + lane] = diag_sum(j + 1);  // the lightest row's warp
-                const int r = j + l;
-                if (r < N) {
-                    sr = s0 + l >= W ? s0 + l - W : s0 + l;
-                    a = widen(band_a(L0.kx, L0.ky, NC, r, l));
-                    if constexpr (FULL) {
-                        for (int u = 0; u < NC - l; ++u) a -= Rs(sr, NC - u) * Rs(s0, NC - l - u);
-                    } else {
-                        for (int tt = (r - NC > 0 ? r - NC : 0); tt < j; ++tt) a -= Rs(sr, r - tt) * Rs(s0, j - tt);
-                    }
-                }
-            } else {
-                v = h2;  // forward substitution, f = 1
-#pragma unroll
-                for (int q = 1; q <= NC; ++q) {
-                    if (!FULL && q > j) break;
-                    v -= Rs(s0, q) * win[q - 1];
-                }
-            }
-            __syncthreads();
-            const double rl = Rs(s0, 0);
-            if (warp == 0) {
-                if (live) {
-#pragma unroll
-                    for (int e = 0; e <= NC; ++e) {
-                        if (!FULL && e > j) break;
-                        fac[static_cast<size_t>(j * W + e) * cs + i] = Rs(s0, e);
-                        if constexpr (MX) f32[static_cast<size_t>(j * W + e) * cs + i] = narrow(Rs(s0, e));
-                    }
-                }
-            } else if (warp <= NC) {
-                if (j + l < N) Rs(sr, l) = a * rl;
-            } else {
-                const double yj = v * rl;
-                ys[j * 32 + lane] = yj;
-#pragma unroll
-                for (int q = NC - 1; q > 0; --q) win[q] = win[q - 1];
-                win[0] = yj;
-            }
-            __syncthreads();
-        };
-        for (int j = 0; j < NC; ++j) step(j, std::false_type());
-        for (int j = NC; j < N; ++j) step(j, std::true_type());
-        if (warp == NC + 1) {
-            // backward: x_r = (y_r - sum_q L(r+q, r) x_(r+q)) / L(r, r), win[q - 1] = x_(r+q)
-            double* x = (MX || A.refine) ? L0.u64 : reinterpret_cast<double*>(L0.u);
-#pragma unroll
-            for (int q = 0; q < NC; ++q) win[q] = 0.0;
-            for (int r = N - 1; r >= 0; --r) {
-                double v = ys[r * 32 + lane];
-#pragma unroll
-                for (int q = 1; q <= NC; ++q)
-                    if (r + q < N) v -= fac[static_cast<size_t>((r + q) * W + q) * cs + si] * win[q - 1];
-                const double xr = v * fac[static_cast<size_t>(r * W) * cs + si];
-                ys[r * 32 + lane] = xr;
-                if (live) {
-                    x[r] = xr;
-                    if constexpr (MX) reinterpret_cast<float*>(L0.u)[r] = narrow(xr);  // FP32 copy for the first FMG interpolation
-                }
-#pragma unroll
-                for (int q = NC - 1; q > 0; --q) win[q] = win[q - 1];
-                win[0] = xr;
-            }
-            double F0;
-            if (A.qoi == MLQMC_QOI_MEAN) {
-                double acc = 0.0;
-                for (int r = 0; r < N; ++r) acc += ys[r * 32 + lane];
-                F0 = acc / static_cast<double>(N);
-            } else {
-                constexpr int m = NC / 2;
-                F0 = 0.25 * (ys[((m - 1) * NC + (m - 1)) * 32 + lane] + ys[((m - 1) * NC + m) * 32 + lane] +
-                             ys[(m * NC + (m - 1)) * 32 + lane] + ys[(m * NC + m) * 32 + lane]);
-            }
-            if (live) A.F[static_cast<size_t>(i) * A.n_levels] = F0;
-        }
-        __syncthreads();
+    const Lv<T> L0 = view<T>(A, 0, si);
+    for (int r = tl; r < N; r += Gm::SEG) {
+        S[Gm::oD + r] = level0_diag(L0.kx, L0.ky, NC, r);
+        S[Gm::oA + 2 * r] = widen(band_a(L0.kx, L0.ky, NC, r, 1));
+        S[Gm::oA + 2 * r + 1] = r >= NC ? widen(band_a(L0.kx, L0.ky, NC, r, NC)) : 0.0;
     }
+    __syncwarp();
+    // LPR = 4: group (p + 2) mod 4 of row slot p holds its diagonal, group (p + 1) mod 4 its
+    // right-hand side: never the group of the column being eliminated when the slot is the pivot
+    const int gd = LPR == 1 ? 0 : (p + 2) % LPR;
+    double off[KR];  // column c of the lane's row, c mod NC = g + LPR k
+    double X, V = 0.0;  // diagonal or right-hand side (LPR = 1: diagonal and right-hand side)
+    auto reset = [&](int r) {  // row r enters the window
+        const bool in = r < N;
+        const int rr = in ? r : 0;
+#pragma unroll
+        for (int k = 0; k < KR; ++k) {
+            const int cm = g + LPR * k;
+            double a = 0.0;
+            if (cm == (r + NC - 1) % NC) a = S[Gm::oA + 2 * rr];
+            if (cm == r % NC) a = S[Gm::oA + 2 * rr + 1];
+            off[k] = in ? a : 0.0;
+        }
+        const double d = S[Gm::oD + rr];
+        if constexpr (LPR == 1) {
+            X = d;
+            V = h2;
+        } else {
+            X = g == gd ? d : h2;
+        }
+    };
+    reset(p);
+    for (int j0 = 0; j0 < N; j0 += NC) {
+#pragma unroll
+        for (int sj = 0; sj < NC; ++sj) {
+            const int j = j0 + sj;
+            constexpr int L1 = LPR - 1;
+            const int gc = sj & L1, kc = sj / LPR;        // group and register of the column being eliminated
+            const int ld = LPR == 1 ? 0 : (sj + 2) % LPR, lv = LPR == 1 ? 0 : (sj + 1) % LPR;
+            const double d = __shfl_sync(0xffffffffu, X, t0 + sj * LPR + ld);
+            const double rl = rsqrt64(d);
+            double yj;
+            double Lm;
+            if constexpr (LPR == 1) {
+                const double vj = __shfl_sync(0xffffffffu, V, t0 + sj);
+                if (p == sj) reset(j + NC);
+                Lm = off[kc] * rl;
+                yj = vj * rl;
+            } else {
+                const double xo = X;
+                if (p == sj) reset(j + NC);
+                Lm = ((p == sj && g == lv) ? xo : off[kc]) * rl;  // one multiplication: column j and y_j
+                yj = __shfl_sync(0xffffffffu, Lm, t0 + sj * LPR + lv);
+            }
+            const double Lr = LPR == 1 ? Lm : __shfl_sync(0xffffffffu, Lm, t0 + p * LPR + gc);
+#pragma unroll
+            for (int k = 0; k < KR; ++k) {
+                const int cm = g + LPR * k;  // row slot of column c
+                if (LPR == 1 && cm == sj) continue;
+                const double Lc = __shfl_sync(0xffffffffu, Lm, t0 + (cm < NC ? cm : 0) * LPR + gc);
+                if (cm != sj) off[k] = fma(-Lr, Lc, off[k]);
+            }
+            if constexpr (LPR == 1) {
+                X = fma(-Lr, Lr, X);
+                V = fma(-Lr, yj, V);
+            } else {
+                X = fma(-Lr, g == gd ? Lr : yj, X);
+            }
+            if (work && g == gc) S[Gm::oL + j * NC + p] = Lr;
+            if (tl == 0) {
+                S[Gm::oR + j] = rl;
+                S[Gm::oY + j] = yj;
+            }
+        }
+    }
+    __syncwarp();
+    // the factor to global memory in one pass (inside the loop its address
+    // arithmetic and, mixed forms, the rounding to FP32 sat on the critical path)
+    if (live) {
+        auto put = [&](int q, double v) {
+            if constexpr (MX) f32[static_cast<size_t>(q) * cs + i] = narrow(v);
+            else fac[static_cast<size_t>(q) * cs + i] = v;
+        };
+        for (int q = tl; q < N * NC; q += Gm::SEG) {  // column j, row slot q mod NC: row j + l
+            const int j = q / NC, l = (q - j * NC + NC - j % NC) % NC;
+            const int lr = l ? l : NC;
+            if (j + lr < N) put((j + lr) * W + lr, S[Gm::oL + q]);
+        }
+        for (int j = tl; j < N; j += Gm::SEG) put(j * W, S[Gm::oR + j]);
+    }
+    __syncwarp();
+    // backward substitution: lane p < NC (LPR lanes of a slot alike) keeps the
+    // pending value of the row of slot p; row r's solution updates rows r-1..r-NC
+    double v = S[Gm::oY + N - NC + p];
+    for (int r0 = N - NC; r0 >= 0; r0 -= NC) {
+#pragma unroll
+        for (int sr = NC - 1; sr >= 0; --sr) {
+            const int r = r0 + sr;
+            const int c = p < sr ? r0 + p : r0 + p - NC;  // the slot's row below r (slot sr: row r - NC enters)
+            const double Lc = c >= 0 ? S[Gm::oL + c * NC + sr] : 0.0;
+            const double xr = __shfl_sync(0xffffffffu, v, t0 + sr * LPR) * S[Gm::oR + r];
+            if (p == sr) v = c >= 0 ? S[Gm::oY + c] : 0.0;
+            v = fma(-Lc, xr, v);
+            if (tl == 0) S[Gm::oY + r] = xr;
+        }
+    }
+    __syncwarp();
+    double* x = (MX || A.refine) ? L0.u64 : reinterpret_cast<double*>(L0.u);
+    if (live)
+        for (int r = tl; r < N; r += Gm::SEG) {
+            x[r] = S[Gm::oY + r];
+            if constexpr (MX) reinterpret_cast<float*>(L0.u)[r] = narrow(S[Gm::oY + r]);  // FP32 copy for the first FMG interpolation
+        }
+    double F0;
+    if (A.qoi == MLQMC_QOI_MEAN) {
+        constexpr int Q = Gm::SEG >= 16 ? 1 : 16 / Gm::SEG;  // partial sums per lane: c = tl + SEG q
+        double s[Q];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int c = (tl & 15) + Gm::SEG * q;
+            s[q] = S[Gm::oY + c];
+            for (int r = 16 + c; r < N; r += 16) s[q] += S[Gm::oY + r];
+        }
+#pragma unroll
+        for (int w = Q / 2; w > 0; w >>= 1)
+#pragma unroll
+            for (int q = 0; q < w; ++q) s[q] += s[q + w];
+        double acc = s[0];
+#pragma unroll
+        for (int w = Gm::SEG >= 16 ? 8 : Gm::SEG / 2; w > 0; w >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, w);
+        F0 = acc / static_cast<double>(N);
+    } else {
+        constexpr int m = NC / 2;
+        const double* y = S + Gm::oY;
+        F0 = 0.25 * (y[(m - 1) * NC + (m - 1)] + y[(m - 1) * NC + m] + y[m * NC + (m - 1)] + y[m * NC + m]);
+    }
+    if (live && tl == 0) A.F[static_cast<size_t>(i) * A.n_levels] = F0;
 }
 
 template <int NC>
@@ -1809,8 +1877,32 @@ mlqmc_status last_error()
     return ok(cudaGetLastError()) ? MLQMC_OK : MLQMC_ERR_CUDA;
 }
 
-// Calls with fewer level-0 samples than this take kb_level0_split.
-constexpr int kLevel0SplitBelow = 16384;
+// Which level-0 kernel a call takes, by its samples. Four lanes per window row
+// (a warp per sample at n0 = 8) has the shortest chain but pays nine FP64 warp
+// instructions per sample and column; one lane per row pays sixteen for 32/n0
+// samples; one thread per sample about 75 for 32 samples, in one long chain.
+// Microseconds per call measured at n0 = 8, FP64 form (four lanes / one lane /
+// one thread): 16 samples 47 / 61 / 219, 1,024: 55 / 62 / 251, 2,048: 96 / 63 /
+// 252, 8,192: 358 / 175 / 255, 16,368: 713 / 337 / 281; at n0 = 4 2,048: 19 / 18 / 39,
+// 16,384: 92 / 37 / 43, 32,768: 171 / 73 / 55. The other sides have no
+// thread-per-sample kernel in registers and shared memory (n0 = 6: one lane 159,
+// one thread 181 at 16,384, 306 / 269 at 32,768).
+constexpr int kLevel0FourLanes = 1280;
+constexpr int level0_one_thread_from(int n0) { return n0 == 8 ? 13000 : 24000; }
+
+// Lanes per window row of the call's level-0 kernel; 0: one thread per sample.
+int level0_lanes(int n0, int B)
+{
+    if (n0 > 10 || n0 < 4 || B >= level0_one_thread_from(n0)) return 0;
+    return B < kLevel0FourLanes && 4 * n0 <= 32 ? 4 : 1;
+}
+
+template <typename T, bool MX, int NC, int LPR>
+void launch_lanes(const FmgArgs& A, int B, cudaStream_t st)
+{
+    using Gm = L0Geom<NC, LPR>;
+    kb_level0_lanes<T, MX, NC, LPR><<<(B + Gm::SPW - 1) / Gm::SPW, 32, Gm::bytes, st>>>(A, B);
+}
 
 // Level-0 factor, exact solve and F_0 of samples 0..B-1.
 mlqmc_status launch_level0(mlqmc_ctx* c, const FmgArgs& A, int B, cudaStream_t st)
@@ -1838,18 +1930,24 @@ mlqmc_status launch_level0(mlqmc_ctx* c, const FmgArgs& A, int B, cudaStream_t s
         per_sm = std::max(1, per_sm);
     }
     const int g64 = std::max(1, std::min((B + 63) / 64, c->sm_count * per_sm));
-    // few samples: one thread per sample would leave most SM sub-partitions
-    // idle, each warp's FP64 chain alone setting the time; split every step
-    // of a group of 32 samples over the warps of a CTA instead (same results)
-    const int g32 = (B + 31) / 32;
-    if (B < kLevel0SplitBelow && (c->p.coarse_cells == 8 || c->p.coarse_cells == 4)) {
-        if (c->p.coarse_cells == 8) {
-            if (is_mixed(c->p)) kb_level0_split<float, true, 8><<<g32, 32 * 10, 0, st>>>(A, B);
-            else kb_level0_split<double, false, 8><<<g32, 32 * 10, 0, st>>>(A, B);
-        } else {
-            if (is_mixed(c->p)) kb_level0_split<float, true, 4><<<g32, 32 * 6, 0, st>>>(A, B);
-            else kb_level0_split<double, false, 4><<<g32, 32 * 6, 0, st>>>(A, B);
+    const int n0c = c->p.coarse_cells;
+    const int lanes = level0_lanes(n0c, B);
+    const bool mx = is_mixed(c->p);
+    auto by_lanes = [&](auto nc) {
+        constexpr int NC = decltype(nc)::value;
+        if constexpr (NC * 4 <= 32) {
+            if (lanes == 4) return mx ? launch_lanes<float, true, NC, 4>(A, B, st) : launch_lanes<double, false, NC, 4>(A, B, st);
         }
+        mx ? launch_lanes<float, true, NC, 1>(A, B, st) : launch_lanes<double, false, NC, 1>(A, B, st);
+    };
+    if (lanes && n0c == 8) {
+        by_lanes(std::integral_constant<int, 8>());
+    } else if (lanes && n0c == 4) {
+        by_lanes(std::integral_constant<int, 4>());
+    } else if (lanes && n0c == 6) {
+        by_lanes(std::integral_constant<int, 6>());
+    } else if (lanes && n0c == 10) {
+        by_lanes(std::integral_constant<int, 10>());
     } else if (c->p.coarse_cells == 8) {
         if (is_mixed(c->p)) kb_level0_fixed<float, true, 8><<<g64, 64, level0_smem<8>(), st>>>(A, B);
         else kb_level0_fixed<double, false, 8><<<g64, 64, level0_smem<8>(), st>>>(A, B);
@@ -3303,6 +3401,7 @@ mlqmc_status round_graph(mlqmc_ctx* c, int count, const int* Bt, int Lmax, doubl
         key.push_back(Bt[t] > 0 ? smoother_for(c, t, Bt[t]) : -1);
         key.push_back(Bt[t] > 0 ? kl_nt_for(c, t, Bt[t]) : 0);
     }
+    key.push_back(level0_lanes(c->p.coarse_cells, Bt[0]));
     key.push_back(d_F ? 1 : 0);
     key.push_back(d_sums ? 1 : 0);
     // an instantiated graph may still be running the previous call
