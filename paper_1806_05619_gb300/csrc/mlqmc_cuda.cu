@@ -24,6 +24,7 @@
 #include <vector>
 
 #include "fmg_device.cuh"
+#include "fmg_small.h"
 #include "mlqmc_internal.h"
 #include "rbgs_stream.h"
 #include "rbgs_tma.h"
@@ -2305,6 +2306,84 @@ mlqmc_status smooth_whole(mlqmc_ctx* c, const FmgArgs& A, int t, int B, int nswe
     return mlqmc_whole::launch(A, t, n, B, nsweeps, ones, first, pre, post, zin, f64, st) ? MLQMC_OK : MLQMC_ERR_CUDA;
 }
 
+// FP64 form: calls with fewer samples on a level than this take its one-launch
+// kernels. FP64 issue bounds the sweeps either way; one launch saves the
+// launches' latency and, past these counts, loses more to its barriers.
+// Microseconds of a call, per level / in one launch: n0 = 8, 32 x 32: 16 samples
+// 499 / 186, 1,024: 895 / 796, 2,048: 1,273 / 1,243, 4,096: 2,122 / 2,332; n0 = 4, 32 x 32: 16:
+// 400 / 187, 256: 445 / 261, 1,024: 670 / 748; n0 = 6, 48 x 48: 1,024: 2,239 / 1,822,
+// 2,048: 3,281 / 3,493.
+constexpr int small_f64_below(int n0) { return n0 == 4 ? 512 : 2048; }
+
+// Largest level up to t_max whose V-cycle part runs in one launch per sample
+// (fmg_small.cuh) for calls with B(t) samples on level t: the levels up to 64
+// cells per side whose smoother is the one that kernel restates (a forced
+// other one keeps its per-level launches); 0: none.
+template <typename Count>
+int small_top(const mlqmc_ctx* c, int t_max, Count B)
+{
+    const bool f64 = !is_mixed(c->p);
+    if (c->p.nu1 < 1 || c->p.nu2 < 1) return 0;
+    int top = 0;
+    for (int t = 1; t <= t_max && t <= mlqmc_small::top_level(c->p.coarse_cells, c->p.n_levels, f64); ++t) {
+        const int own = mlqmc_whole::supported(c->p.coarse_cells << t, f64)
+                            ? MLQMC_SMOOTHER_WHOLE
+                            : (f64 ? MLQMC_SMOOTHER_GS : MLQMC_SMOOTHER_TILE);
+        if (smoother_for(c, t, B(t)) != own || (f64 && B(t) >= small_f64_below(c->p.coarse_cells))) break;
+        top = t;
+    }
+    return top;
+}
+
+// Algorithmic work of one V-cycle on levels top..0 (faces, right-hand sides
+// and factor in, the top iterate out; the levels' sweeps and transfers).
+template <typename T>
+Work small_work(const mlqmc_ctx* c, int top, double B, double cycles)
+{
+    const double N0 = cells_of(c, 0), n0 = c->p.coarse_cells, es = sizeof(T);
+    double bytes = es * (N0 * (n0 + 1.0) + 2.0 * cells_of(c, top)), flops = 4.0 * N0 * n0;
+    for (int t = 1; t <= top; ++t) {
+        bytes += es * 2.0 * faces_of(c, t);
+        flops += cells_of(c, t) * (10.0 * (c->p.nu1 + c->p.nu2) + 19.0);
+    }
+    return work_of<T>(B * bytes, B * cycles * flops);
+}
+
+// Levels top..0 of a V-cycle for samples 0..B-1 in one launch.
+template <typename T>
+mlqmc_status small_vcycle(mlqmc_ctx* c, const FmgArgs& A, int top, int B, cudaStream_t st)
+{
+    LevelTag lt(c, top);
+    const bool f64 = sizeof(T) == 8;
+    const mlqmc_small::Plan P = mlqmc_small::make_plan(c->p.coarse_cells, top, f64, false, false);
+    Timed tm(c, kProfSmallV, st, small_work<T>(c, top, B, 1.0));
+    return (f64 ? mlqmc_small::vcycle_f64(A, P, B, st) : mlqmc_small::vcycle_f32(A, P, B, st)) ? MLQMC_OK : MLQMC_ERR_CUDA;
+}
+
+// FMG stages 1..top in one launch per class of samples whose FMG ends on, or
+// goes on past, level top, top - 1, ..., 1 (ranks are by finest level).
+template <typename T>
+mlqmc_status small_stages(mlqmc_ctx* c, const FmgArgs& A, const int* Bt, int top, bool keep, cudaStream_t st)
+{
+    const bool f64 = sizeof(T) == 8, conv = !f64 && c->p.refine_rtol > 0.0;
+    for (int t = top; t >= 1; --t) {
+        mlqmc_small::Stages S{};
+        S.i0 = t == top ? 0 : Bt[t + 1];
+        S.keep = keep ? 1 : 0;
+        S.thresh = conv ? c->p.refine_rtol : 0.0;
+        S.max_iter = c->p.refine_max_iter;
+        S.iters = c->d_iters + MLQMC_MAX_LEVELS;
+        const int count = Bt[t] - S.i0;
+        if (count <= 0) continue;
+        LevelTag lt(c, t);
+        const mlqmc_small::Plan P = mlqmc_small::make_plan(c->p.coarse_cells, t, f64, true, conv);
+        Timed tm(c, kProfSmallV, st, small_work<T>(c, t, count, c->p.mu0 * 1.4));
+        if (!(f64 ? mlqmc_small::stages_f64(A, P, S, count, st) : mlqmc_small::stages_f32(A, P, S, count, st)))
+            return MLQMC_ERR_CUDA;
+    }
+    return MLQMC_OK;
+}
+
 // Whether the pre-smoother of level t starts a correction from zero without
 // reading u (so the V-cycle need not clear u first).
 template <typename T>
@@ -2357,7 +2436,9 @@ template <typename T>
 mlqmc_status vcycle_batched(mlqmc_ctx* c, FmgArgs& A, int t_top, int B, bool ones, cudaStream_t st,
                             bool top_zero = false)
 {
-    for (int t = t_top; t >= 1; --t) {
+    // the levels below t_top that fit one launch per sample, else the coarse solve alone
+    const int small = small_top(c, t_top - 1, [B](int) { return B; });
+    for (int t = t_top; t > small; --t) {
         const int top_ones = (t == t_top && ones) ? 1 : 0;
         // a correction level (and, top_zero, the top level: the first cycle of a
         // refinement step) starts from zero: cleared here, or by its smoother
@@ -2366,13 +2447,15 @@ mlqmc_status vcycle_batched(mlqmc_ctx* c, FmgArgs& A, int t_top, int B, bool one
         if (zero_entry && !zin && zero_u(c, t, B, st) != MLQMC_OK) return MLQMC_ERR_CUDA;
         if (presmooth_restrict<T>(c, A, t, B, top_ones, st, zin) != MLQMC_OK) return MLQMC_ERR_CUDA;
     }
-    {
+    if (small > 0) {
+        if (small_vcycle<T>(c, A, small, B, st) != MLQMC_OK) return MLQMC_ERR_CUDA;
+    } else {
         const double N0 = cells_of(c, 0), n0 = c->p.coarse_cells, es = sizeof(T);
         Timed tm(c, kProfSmallV, st, work_of<T>(B * es * (N0 * (n0 + 1.0) + 2.0 * N0), B * 4.0 * N0 * n0));
         LevelTag lt(c, 0);
         launch_coarse<T>(c, A, B, st);
     }
-    for (int t = 1; t <= t_top; ++t) {
+    for (int t = small + 1; t <= t_top; ++t) {
         const int top_ones = (t == t_top && ones) ? 1 : 0;
         if (correct_postsmooth<T>(c, A, t, B, top_ones, st) != MLQMC_OK) return MLQMC_ERR_CUDA;
     }
@@ -2525,7 +2608,21 @@ mlqmc_status fmg_stages(mlqmc_ctx* c, FmgArgs& A, const int* Bt, int Lmax, doubl
     // solution output); otherwise, on the TMA interpolation levels, the
     // interpolant itself travels in FP32 (interp32: in the level's field array)
     const int keep64 = (d_usol != nullptr || c->p.qoi != MLQMC_QOI_MEAN) ? 1 : 0;
-    for (int t = 1; t <= Lmax; ++t) {
+    // the small levels' stages in one launch (the converged FP64 form keeps them level by level)
+    const int small = (MX || !refine) ? small_top(c, Lmax, [Bt](int t) { return Bt[t]; }) : 0;
+    if (small > 0) {
+        const mlqmc_status s = small_stages<T>(c, A, Bt, small, d_usol != nullptr, st);
+        if (s != MLQMC_OK) return s;
+        for (int t = 1; d_usol && t <= small; ++t) {
+            LevelTag lt(c, t);
+            const int64_t n = c->p.coarse_cells << t;
+            Timed tm(c, kProfReduce, st, work_of<double>((8.0 + (refine ? 8.0 : sizeof(T))) * cells_of(c, t), 0.0));
+            if (refine) kb_u_out<T, true><<<grid_for(c, n * n), 256, 0, st>>>(A, t, d_usol + uoff);
+            else kb_u_out<T, false><<<grid_for(c, n * n), 256, 0, st>>>(A, t, d_usol + uoff);
+            uoff += static_cast<size_t>(n) * n;
+        }
+    }
+    for (int t = small + 1; t <= Lmax; ++t) {
         const int B = Bt[t];
         if (B == 0) break;
         LevelTag lt(c, t);
@@ -2652,8 +2749,11 @@ mlqmc_status tune_smoothers(mlqmc_ctx* c)
     mlqmc_status res = MLQMC_OK;
     const int all[4] = {MLQMC_SMOOTHER_GS, MLQMC_SMOOTHER_WHOLE, MLQMC_SMOOTHER_STREAM, MLQMC_SMOOTHER_TMA};
     int large_best[MLQMC_MAX_LEVELS] = {};
+    // the levels that run in one launch per sample need no choice
+    const int fused = small_top(c, c->p.n_levels - 1, [](int) { return 1; });
     for (int t = 1; t < c->p.n_levels && res == MLQMC_OK; ++t)
     for (int cls = 1; cls >= 0 && res == MLQMC_OK; --cls) {  // large batches, then small ones
+        if (t <= fused) continue;
         int cands[4], nc = 0;
         for (int k : all)
             if ((f64 || k != MLQMC_SMOOTHER_GS) && smoother_fits(c, k, t)) cands[nc++] = k;
@@ -3196,7 +3296,8 @@ extern "C" mlqmc_status mlqmc_create(const mlqmc_problem* p, int64_t max_samples
     size_t free_b = 0, total_b = 0;
     cudaMemGetInfo(&free_b, &total_b);
     c->pool_budget = std::min<size_t>(free_b / 2, static_cast<size_t>(192) << 30);
-    if (!mlqmc_tma::prepare() || !mlqmc_whole::prepare() || !mlqmc_resid::prepare()) {
+    if (!mlqmc_tma::prepare() || !mlqmc_whole::prepare() || !mlqmc_resid::prepare() ||
+        !(is_mixed(*p) ? mlqmc_small::prepare_f32() : mlqmc_small::prepare_f64())) {
         free_ctx(c);
         return MLQMC_ERR_CUDA;
     }
@@ -3402,6 +3503,7 @@ mlqmc_status round_graph(mlqmc_ctx* c, int count, const int* Bt, int Lmax, doubl
         key.push_back(Bt[t] > 0 ? kl_nt_for(c, t, Bt[t]) : 0);
     }
     key.push_back(level0_lanes(c->p.coarse_cells, Bt[0]));
+    for (int t = 1; t <= Lmax; ++t) key.push_back(t == Lmax || Bt[t] > Bt[t + 1] ? 1 : 0);  // launches of the small stages
     key.push_back(d_F ? 1 : 0);
     key.push_back(d_sums ? 1 : 0);
     // an instantiated graph may still be running the previous call

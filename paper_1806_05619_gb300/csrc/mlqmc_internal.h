@@ -62,7 +62,7 @@ enum ProfKind {
     kProfSynth = 2,    // batched KL field, faces, inverse diagonal
     kProfSmooth = 3,   // batched red-black sweeps
     kProfTransfer = 4, // batched residual/restriction, prolongation, FP64 refinement updates
-    kProfSmallV = 5,   // coarse solves of the V-cycles (one thread per sample)
+    kProfSmallV = 5,   // small levels in one launch (their FMG stages, the V-cycles' part on them), coarse solves
     kProfReduce = 6,   // QoI, norms, reuse sums, outputs
     kProfKlTc = 7,     // KL contraction on the tensor cores
     kProfKinds = 8
