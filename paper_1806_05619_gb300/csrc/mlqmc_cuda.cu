@@ -29,6 +29,7 @@
 #include "rbgs_stream.h"
 #include "rbgs_tma.h"
 #include "resid_tma.h"
+#include "resnorm_pairs.h"
 #include "ptx_async.cuh"
 #include "rbgs_whole.h"
 #include "matern_nystrom.h"
@@ -1272,19 +1273,25 @@ __global__ void __launch_bounds__(256) kb_resnorm_part(FmgArgs A, int t, int B, 
     }
 }
 
-// norms[i] = sqrt of the sum of sample i's P partial sums (in chunk order),
-// active[i] = (norm_i > thresh); *count = number of active samples.
-__global__ void kb_norm_flags(const double* part, int P, double* norms, int* active, int B, double thresh, int* count)
+// norms[i] = sqrt of the sum of sample i's P partial sums (a warp per sample, in
+// a fixed order: one thread's chain of P dependent FP64 adds took longer than
+// the rest of a small pass), active[i] = (norm_i > thresh); *count = number of
+// active samples.
+__global__ void __launch_bounds__(256) kb_norm_flags(const double* part, int P, double* norms, int* active, int B,
+                                                     double thresh, int* count)
 {
-    GRID_STRIDE(i, B)
-    {
+    const int lane = threadIdx.x & 31;
+    for (int i = blockIdx.x * 8 + (threadIdx.x >> 5); i < B; i += gridDim.x * 8) {
         double sum = 0.0;
-        for (int q = 0; q < P; ++q) sum += part[static_cast<size_t>(i) * P + q];
-        const double nr = sqrt(sum);
-        norms[i] = nr;
-        const int a = nr > thresh ? 1 : 0;
-        active[i] = a;
-        if (a) atomicAdd(count, 1);
+        for (int q = lane; q < P; q += 32) sum += part[static_cast<size_t>(i) * P + q];
+        sum = team_sum(WarpTeam{}, sum, nullptr);
+        if (lane == 0) {
+            const double nr = sqrt(sum);
+            norms[i] = nr;
+            const int a = nr > thresh ? 1 : 0;
+            active[i] = a;
+            if (a) atomicAdd(count, 1);
+        }
     }
 }
 
@@ -2462,22 +2469,49 @@ mlqmc_status vcycle_batched(mlqmc_ctx* c, FmgArgs& A, int t_top, int B, bool one
     return last_error();
 }
 
+// Partial residual sums per sample on level t: the tiles of the pair kernel
+// (mixed forms), or chunks of about 8192 cells.
+int norm_chunks(const mlqmc_ctx* c, int t)
+{
+    const int n = c->p.coarse_cells << t;
+    if (is_mixed(c->p) && mlqmc_resnorm::supported(n)) return mlqmc_resnorm::chunks(n);
+    return std::max(1, static_cast<int>(static_cast<int64_t>(n) * n / 8192));
+}
+
+// Residual (into bc) and its partial norms on level t; active: null on a
+// level's first pass, else the flags of the pass before (a sample that had
+// converged is as it was).
+template <typename T>
+mlqmc_status resnorm(mlqmc_ctx* c, const FmgArgs& A, int t, int B, int P, const int* active, cudaStream_t st)
+{
+    const int n = c->p.coarse_cells << t;
+    const double es = sizeof(T), Mc = cells_of(c, t), Fc = faces_of(c, t);
+    if constexpr (sizeof(T) == 4) {
+        if (mlqmc_resnorm::supported(n)) {
+            Work w = work_of<double>(B * (8.0 * Mc + es * (2.0 * Fc + Mc) + 8.0), B * 2.0 * Mc);
+            w.f32 = B * 12.0 * Mc;
+            Timed tm(c, kProfReduce, st, w);
+            return mlqmc_resnorm::launch(A, t, n, B, c->d_part, active, c->sm_count, st) ? MLQMC_OK : MLQMC_ERR_CUDA;
+        }
+    }
+    Timed tm(c, kProfReduce, st, work_of<double>(B * (8.0 * Mc + es * (2.0 * Fc + Mc) + 8.0), B * 12.0 * Mc));
+    const int grid = static_cast<int>(std::min<int64_t>(static_cast<int64_t>(B) * P, c->sm_count * 8));
+    kb_resnorm_part<T><<<grid, 256, 0, st>>>(A, t, B, P, c->d_part);
+    return last_error();
+}
+
 // Residual norms, flags and the loop decision of one refinement pass on level t.
 template <typename T>
-mlqmc_status norms_and_ctl(mlqmc_ctx* c, const FmgArgs& A, int t, int B, int P, cudaGraphConditionalHandle h,
-                           cudaStream_t st)
+mlqmc_status norms_and_ctl(mlqmc_ctx* c, const FmgArgs& A, int t, int B, int P, const int* active,
+                           cudaGraphConditionalHandle h, cudaStream_t st)
 {
-    const double es = sizeof(T), Mc = cells_of(c, t), Fc = faces_of(c, t);
-    {
-        Timed tm(c, kProfReduce, st, work_of<double>(B * (8.0 * Mc + es * (2.0 * Fc + Mc) + 8.0), B * 12.0 * Mc));
-        const int grid = static_cast<int>(std::min<int64_t>(static_cast<int64_t>(B) * P, c->sm_count * 8));
-        kb_resnorm_part<T><<<grid, 256, 0, st>>>(A, t, B, P, c->d_part);
-    }
+    const mlqmc_status s = resnorm<T>(c, A, t, B, P, active, st);
+    if (s != MLQMC_OK) return s;
     {
         const int64_t n = c->p.coarse_cells << t;
         Timed tm(c, kProfReduce, st, work_of<double>(B * (8.0 * P + 12.0), B * 1.0 * P), 2);
-        kb_norm_flags<<<grid_for(c, B), 256, 0, st>>>(c->d_part, P, c->d_norms, c->d_active, B,
-                                                      c->p.refine_rtol * n, c->d_count);
+        kb_norm_flags<<<grid_for(c, B, 8), 256, 0, st>>>(c->d_part, P, c->d_norms, c->d_active, B,
+                                                         c->p.refine_rtol * n, c->d_count);
         k_loop_ctl<<<1, 1, 0, st>>>(h, c->d_count, c->d_iters + t, c->p.refine_max_iter, c->d_status);
     }
     return last_error();
@@ -2507,7 +2541,7 @@ mlqmc_status converge_device(mlqmc_ctx* c, FmgArgs& A, int t, int B, int P, cuda
     if (!ok(cudaMemsetAsync(c->d_count, 0, sizeof(int), st)) ||
         !ok(cudaMemsetAsync(c->d_iters + t, 0, sizeof(int), st)))
         return MLQMC_ERR_CUDA;
-    mlqmc_status s = norms_and_ctl<T>(c, A, t, B, P, h, st);
+    mlqmc_status s = norms_and_ctl<T>(c, A, t, B, P, nullptr, h, st);
     if (s != MLQMC_OK) return s;
     if (!ok(cudaStreamGetCaptureInfo(st, &cs, nullptr, &cg, &deps, &edges, &nd))) return MLQMC_ERR_CUDA;
     cudaGraphNodeParams np{};
@@ -2529,7 +2563,7 @@ mlqmc_status converge_device(mlqmc_ctx* c, FmgArgs& A, int t, int B, int P, cuda
         kb_update64<T><<<grid_for(c, B * n * n), 256, 0, bs>>>(A, t, B);
     }
     A.active = nullptr;
-    if (s == MLQMC_OK) s = norms_and_ctl<T>(c, A, t, B, P, h, bs);
+    if (s == MLQMC_OK) s = norms_and_ctl<T>(c, A, t, B, P, c->d_active, h, bs);
     G.in_body = false;
     cudaGraph_t body_out = nullptr;
     const bool ended = ok(cudaStreamEndCapture(bs, &body_out));
@@ -2547,9 +2581,8 @@ mlqmc_status converge_batched(mlqmc_ctx* c, FmgArgs& A, int t, int B, cudaStream
 {
     LevelTag lt(c, t);
     const int64_t n = c->p.coarse_cells << t;
-    const double es = sizeof(T), Mc = cells_of(c, t), Fc = faces_of(c, t);
-    // chunks of about 8192 cells per CTA (this path is never graph-captured: the buffer may grow here)
-    const int P = static_cast<int>(std::max<int64_t>(1, n * n / 8192));
+    const double es = sizeof(T), Mc = cells_of(c, t);
+    const int P = norm_chunks(c, t);  // outside a round's capture (prepare_round made room) the buffer may grow here
     if (static_cast<int64_t>(B) * P > c->part_cap) {
         cudaFree(c->d_part);
         c->d_part = nullptr;
@@ -2559,16 +2592,13 @@ mlqmc_status converge_batched(mlqmc_ctx* c, FmgArgs& A, int t, int B, cudaStream
     }
     if (c->graph.round_capture) return converge_device<T>(c, A, t, B, P, st);
     for (int it = 0;; ++it) {
-        {
-            Timed tm(c, kProfReduce, st, work_of<double>(B * (8.0 * Mc + es * (2.0 * Fc + Mc) + 8.0), B * 12.0 * Mc));
-            const int grid = static_cast<int>(std::min<int64_t>(static_cast<int64_t>(B) * P, c->sm_count * 8));
-            kb_resnorm_part<T><<<grid, 256, 0, st>>>(A, t, B, P, c->d_part);
-        }
+        const mlqmc_status rs = resnorm<T>(c, A, t, B, P, it > 0 ? c->d_active : nullptr, st);
+        if (rs != MLQMC_OK) return rs;
         if (!ok(cudaMemsetAsync(c->d_count, 0, sizeof(int), st))) return MLQMC_ERR_CUDA;
         {
             Timed tm(c, kProfReduce, st, work_of<double>(B * (8.0 * P + 12.0), B * 1.0 * P));
-            kb_norm_flags<<<grid_for(c, B), 256, 0, st>>>(c->d_part, P, c->d_norms, c->d_active, B,
-                                                          c->p.refine_rtol * n, c->d_count);
+            kb_norm_flags<<<grid_for(c, B, 8), 256, 0, st>>>(c->d_part, P, c->d_norms, c->d_active, B,
+                                                             c->p.refine_rtol * n, c->d_count);
         }
         if (!ok(cudaMemcpyAsync(c->h_count, c->d_count, sizeof(int), cudaMemcpyDeviceToHost, st)) ||
             !ok(cudaStreamSynchronize(st)))
@@ -3467,10 +3497,7 @@ mlqmc_status prepare_round(mlqmc_ctx* c, const int* Bt, int Lmax)
     }
     if (c->p.refine_rtol > 0.0) {
         int64_t need = 0;
-        for (int t = 1; t <= Lmax; ++t) {
-            const int64_t n = c->p.coarse_cells << t;
-            need = std::max<int64_t>(need, static_cast<int64_t>(Bt[t]) * std::max<int64_t>(1, n * n / 8192));
-        }
+        for (int t = 1; t <= Lmax; ++t) need = std::max<int64_t>(need, static_cast<int64_t>(Bt[t]) * norm_chunks(c, t));
         if (need > c->part_cap) {
             cudaDeviceSynchronize();
             cudaFree(c->d_part);
