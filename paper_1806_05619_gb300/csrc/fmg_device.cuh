@@ -31,12 +31,12 @@ struct ArrDesc {
 struct LevelDesc {
     int n;
     ArrDesc u, bc, kx, ky, idiag, k, G, u64, u2;  // u2: ping-pong partner of u for the tiled smoother
-    // dividers of a flat cell index (nc = n / 2, nq = n / 4, Ka the KL groups)
-    FastDiv by_n, by_nc, by_nq, by_nn, by_ncnc, by_nnc, by_nnq, by_kan;
+    // dividers of a flat cell index (nc = n / 2, nq = n / 4)
+    FastDiv by_n, by_nc, by_nq, by_nn, by_ncnc, by_nnc, by_nnq;
 };
 
 // Fill the dividers of level descriptor d (d.n set), on the host.
-inline void set_divisors(LevelDesc& d, int Ka)
+inline void set_divisors(LevelDesc& d)
 {
     const uint32_t n = static_cast<uint32_t>(d.n), nc = n / 2 > 0 ? n / 2 : 1, nq = n / 4 > 0 ? n / 4 : 1;
     d.by_n = FastDiv(n);
@@ -46,7 +46,6 @@ inline void set_divisors(LevelDesc& d, int Ka)
     d.by_ncnc = FastDiv(nc * nc);
     d.by_nnc = FastDiv(n * nc);
     d.by_nnq = FastDiv(n * nq);
-    d.by_kan = FastDiv(static_cast<uint32_t>(Ka > 0 ? Ka : 1) * n);
 }
 
 template <typename T>
@@ -213,17 +212,16 @@ __device__ __forceinline__ double exp64(double x)
 }
 
 // 1/d for a positive normal d in FP64: the hardware's reciprocal estimate
-// refined by two Newton-Raphson steps r <- r + r (1 - d r), each squaring the
-// relative error, which ends within one ulp of the correctly rounded value
-// in six FP64 operations (IEEE division takes about twelve).
+// refined by one step of third order, r <- r + r (e + e^2) with e = 1 - d r,
+// which cubes its relative error (below 2^-20) and ends within one ulp of the
+// correctly rounded value, in three FP64 operations (two Newton-Raphson steps
+// take four, IEEE division about twelve).
 __device__ __forceinline__ double rcp64(double d)
 {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-    double e = fma(-d, r, 1.0);
-    r = fma(r, e, r);
-    e = fma(-d, r, 1.0);
-    return fma(r, e, r);
+    const double e = fma(-d, r, 1.0);
+    return fma(r, fma(e, e, e), r);
 }
 
 // 1/sqrt(d) for a positive normal d in FP64: the hardware's estimate refined
@@ -244,9 +242,16 @@ __device__ __forceinline__ double expT(double x) { return exp64(x); }
 
 // Harmonic mean 2ab/(a+b) of two cell coefficients: FP32 with the hardware
 // reciprocal (__fdividef, within 2 ulp; the coefficients are positive and
-// far from the range where it flushes), FP64 through rcp64.
+// far from the range where it flushes), FP64 through rcp64 of the halved sum
+// (an exponent decrement off the FP64 pipe; exact for coefficients above
+// 2^-1021): six FP64 operations, and NaN where a or b is infinite or NaN, as in
+// the formula.
 __device__ __forceinline__ float hmean(float a, float b) { return __fdividef(2.0f * a * b, a + b); }
-__device__ __forceinline__ double hmean(double a, double b) { return 2.0 * a * b * rcp64(a + b); }
+__device__ __forceinline__ double hmean(double a, double b) 
+{
+    const double s = a + b;
+    return a * b * rcp64(__hiloint2double(__double2hiint(s) - 0x00100000, __double2loint(s)));
+}
 __device__ __forceinline__ float recip(float d) { return 1.0f / d; }
 __device__ __forceinline__ double recip(double d) { return rcp64(d); }
 
@@ -317,13 +322,14 @@ __device__ void synth_level(const TM& tm, const FmgArgs& A, const Lv<T>& L, int 
 }
 
 // Gauss-Seidel update of one cell: u_P = (h^2 b_P + sum_Q k_PQ u_Q) / D_P.
-template <typename T>
+// b == null: b = 1; ONES (FP64): known to be (no product: five operations, not six).
+template <typename T, bool ONES>
 __device__ __forceinline__ void gs_cell(const Lv<T>& L, const T* b, T h2, int i1, int i2)
 {
     const int n = L.n;
     const int p = i2 * n + i1;
     const T* kx = L.kx + i2 * kx_pitch(n);
-    T acc = h2 * (b ? b[p] : T(1));
+    T acc = ONES ? h2 : h2 * (b ? b[p] : T(1));
     if (i1 > 0) acc += kx[i1] * L.u[p - 1];
     if (i1 < n - 1) acc += kx[i1 + 1] * L.u[p + 1];
     if (i2 > 0) acc += L.ky[i2 * n + i1] * L.u[p - n];
@@ -340,7 +346,7 @@ __device__ __forceinline__ void gs_colour(const TM& tm, const Lv<T>& L, const T*
     const T h2 = T(1) / (T(n) * T(n));
     for (int idx = tm.rank(); idx < n * half; idx += tm.size()) {
         const int i2 = idx / half;
-        gs_cell(L, b, h2, 2 * (idx - i2 * half) + ((i2 + colour) & 1), i2);
+        gs_cell<T, false>(L, b, h2, 2 * (idx - i2 * half) + ((i2 + colour) & 1), i2);
     }
     tm.sync();
 }
@@ -360,12 +366,37 @@ __device__ __forceinline__ U apply_h2(const T* kx, const T* ky, const U* u, int 
     return acc;
 }
 
+// h^2 (A u) summed over the four children of a coarse cell, FP64: the fluxes
+// through the four faces between the children cancel exactly (each enters two
+// children's sums with opposite signs), so only the eight outer ones are formed,
+// 16 FP64 operations in place of 32, without the inner ones' rounding. kx, ky, u
+// at the child (0, 0); `pitch` of kx; w, e, s, n: a neighbour on that side exists.
+__device__ __forceinline__ double quad_flux(const double* kx, const double* ky, const double* u, int n, int pitch, bool w,
+                                            bool e, bool s, bool nn)
+{
+    double a = kx[0] * (u[0] - (w ? u[-1] : 0.0));
+    a = fma(kx[pitch], u[n] - (w ? u[n - 1] : 0.0), a);
+    a = fma(kx[2], u[1] - (e ? u[2] : 0.0), a);
+    a = fma(kx[pitch + 2], u[n + 1] - (e ? u[n + 2] : 0.0), a);
+    a = fma(ky[0], u[0] - (s ? u[-n] : 0.0), a);
+    a = fma(ky[1], u[1] - (s ? u[1 - n] : 0.0), a);
+    a = fma(ky[2 * n], u[n] - (nn ? u[2 * n] : 0.0), a);
+    return fma(ky[2 * n + 1], u[n + 1] - (nn ? u[2 * n + 1] : 0.0), a);
+}
+
 // Coarse value (I1, I2) of the restricted residual: mean over the 4 children of b - A u.
 template <typename T>
 __device__ __forceinline__ T resid_restrict_cell(const Lv<T>& F, const T* b, int I1, int I2)
 {
     const int n = F.n;
     const T ih2 = T(n) * T(n);
+    if constexpr (sizeof(T) == 8) {
+        const int o = 2 * I2 * n + 2 * I1, pitch = kx_pitch(n);
+        const double q = quad_flux(F.kx + 2 * I2 * pitch + 2 * I1, F.ky + o, F.u + o, n, pitch, I1 > 0, 2 * I1 + 2 < n,
+                                   I2 > 0, 2 * I2 + 2 < n);
+        const double sb = b ? (b[o] + b[o + 1]) + (b[o + n] + b[o + n + 1]) : 4.0;
+        return 0.25 * fma(-ih2, q, sb);
+    }
     T s = T(0);
 #pragma unroll
     for (int d = 0; d < 4; ++d) {
@@ -406,6 +437,23 @@ __device__ __forceinline__ D prolong_cell(const S* e, int nc, int i1, int i2)
     const D c = o2 ? -c0 : c0;
     const D d = (o1 != o2) ? -d0 : d0;
     return fma(D(0.5625), a, fma(D(0.1875), b + c, D(0.0625) * d));
+}
+
+// The four fine cells of a coarse parent from its 3 x 3 neighbourhood in FP64,
+// the bilinear weights applied along x1, then along x2 (3/4 of the nearer row
+// or column as 3, scaled by 1/16 at the end, which is exact): 14 FP64
+// operations per quad with the addition to u, where prolong_cell's form takes 20.
+__device__ __forceinline__ void prolong_quad64(const double (&E)[3][3], double (&out)[2][2])
+{
+    double r[3][2];
+#pragma unroll
+    for (int y = 0; y < 3; ++y)
+#pragma unroll
+        for (int fx = 0; fx < 2; ++fx) r[y][fx] = fma(3.0, E[y][1], E[y][2 * fx]);
+#pragma unroll
+    for (int fy = 0; fy < 2; ++fy)
+#pragma unroll
+        for (int fx = 0; fx < 2; ++fx) out[fy][fx] = 0.0625 * fma(3.0, r[1][fx], r[2 * fy][fx]);
 }
 
 template <typename S, typename D, bool ADD, typename TM>

@@ -32,12 +32,19 @@ __device__ __forceinline__ T mul_rn(T a, T b)
     else return __dmul_rn(a, b);
 }
 
+// hb + sum_j k_j u_j (hb: the rounded product h^2 b)
+template <typename T>
+__device__ __forceinline__ T gs_sum(T hb, T k0, T u0, T k1, T u1, T k2, T u2, T k3, T u3)
+{
+    return fma(k3, u3, fma(k2, u2, fma(k1, u1, fma(k0, u0, hb))));
+}
+
 // h^2 b + sum_j k_j u_j
 template <typename T, bool HEAD>
 __device__ __forceinline__ T gs_sum(T h2, T b, T k0, T u0, T k1, T u1, T k2, T u2, T k3, T u3)
 {
-    const T a = HEAD ? fma(h2, b, mul_rn(k0, u0)) : fma(k0, u0, mul_rn(h2, b));
-    return fma(k3, u3, fma(k2, u2, fma(k1, u1, a)));
+    if constexpr (!HEAD) return gs_sum(mul_rn(h2, b), k0, u0, k1, u1, k2, u2, k3, u3);
+    return fma(k3, u3, fma(k2, u2, fma(k1, u1, fma(h2, b, mul_rn(k0, u0)))));
 }
 
 // sum_j k_j d_j
@@ -81,16 +88,17 @@ __device__ __forceinline__ void half_sweep(const Level& L, T* S, int colour, boo
         const int x = 2 * m + ((y + colour) & 1);
         const int c0 = y * n + x;
         const T* kr = skx + y * XP;
-        T acc = h2 * (ones ? T(1) : sb[c0]);
+        T acc = h2;  // b = 1: no product
+        if (!ones) acc = mul_rn(h2, sb[c0]);
         if constexpr (!FIRST)
-            acc = gs_sum<T, false>(h2, ones ? T(1) : sb[c0], kr[x], x > 0 ? su[c0 - 1] : T(0), kr[x + 1], x < n - 1 ? su[c0 + 1] : T(0),
+            acc = gs_sum(acc, kr[x], x > 0 ? su[c0 - 1] : T(0), kr[x + 1], x < n - 1 ? su[c0 + 1] : T(0),
                          sky[c0], y > 0 ? su[c0 - n] : T(0), sky[c0 + n], y < n - 1 ? su[c0 + n] : T(0));
         su[c0] = acc * sd[c0];
     }
     __syncthreads();
 }
 
-// bc of level t-1: mean over the 4 children of b - A u.
+// bc of level t-1: mean over the 4 children of b - A u (resid_restrict_cell's arithmetic).
 template <typename T, int NC>
 __device__ __forceinline__ void restrict_residual(const Level& F, const Level& C, T* S, bool ones)
 {
@@ -100,6 +108,14 @@ __device__ __forceinline__ void restrict_residual(const Level& F, const Level& C
     for (int q = threadIdx.x; q < nc * nc; q += blockDim.x) {
         int I2, I1;
         split<NC>(C, false, q, I2, I1);
+        if constexpr (sizeof(T) == 8) {
+            const int o = 2 * I2 * n + 2 * I1;
+            const double qf = quad_flux(skx + 2 * I2 * XP + 2 * I1, sky + o, su + o, n, XP, I1 > 0, I1 < nc - 1, I2 > 0,
+                                        I2 < nc - 1);
+            const double sum = ones ? 4.0 : (sb[o] + sb[o + 1]) + (sb[o + n] + sb[o + n + 1]);
+            S[C.oB + q] = 0.25 * fma(-ih2, qf, sum);
+            continue;
+        }
         T s = T(0);
 #pragma unroll
         for (int d = 0; d < 4; ++d) {
@@ -139,14 +155,26 @@ __device__ __forceinline__ void interpolate(const Level& C, const T* se, T* dst)
             }
         }
         T* f = dst + (2 * I2) * n + 2 * I1;
+        if constexpr (sizeof(T) == 8) {
+            double v[2][2];
+            prolong_quad64(E, v);
 #pragma unroll
-        for (int fy = 0; fy < 2; ++fy)
+            for (int fy = 0; fy < 2; ++fy)
 #pragma unroll
-            for (int fx = 0; fx < 2; ++fx) {
-                const T v = fma(T(0.5625), E[1][1], fma(T(0.1875), E[1][2 * fx] + E[2 * fy][1], T(0.0625) * E[2 * fy][2 * fx]));
-                if constexpr (ADD) f[fy * n + fx] += v;
-                else f[fy * n + fx] = v;
-            }
+                for (int fx = 0; fx < 2; ++fx) {
+                    if constexpr (ADD) f[fy * n + fx] += v[fy][fx];
+                    else f[fy * n + fx] = v[fy][fx];
+                }
+        } else {
+#pragma unroll
+            for (int fy = 0; fy < 2; ++fy)
+#pragma unroll
+                for (int fx = 0; fx < 2; ++fx) {
+                    const T v = fma(T(0.5625), E[1][1], fma(T(0.1875), E[1][2 * fx] + E[2 * fy][1], T(0.0625) * E[2 * fy][2 * fx]));
+                    if constexpr (ADD) f[fy * n + fx] += v;
+                    else f[fy * n + fx] = v;
+                }
+        }
     }
     __syncthreads();
 }

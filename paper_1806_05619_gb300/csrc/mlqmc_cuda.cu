@@ -694,30 +694,46 @@ __device__ __forceinline__ bool inactive(const FmgArgs& A, int i)
     return A.active && !A.active[i];
 }
 
+// The separable modes are even (odd) about the middle of the unit interval for
+// even (odd) index: with HALF the even and the odd part of a sum, formed on the
+// left half, give both halves as their sum and difference, at half the products.
+// The FP64 pipe bounds both kernels on large levels (six levels of 1024..32
+// points x 16 shifts, 100 modes: kb_synth_z 5.27 -> 4.05 ms); below 64 cells per
+// side a call is too small for it to matter and two exponentials per thread take
+// longer than one (32 x 32, ten modes: 4.7 / 3.5 us).
+constexpr int kHalfFrom = 64;
+
 // G[i][a][i2] = sum_{m: a_m = a} sqrt(theta_m) y_m psi_{b_m}(x2)
-template <typename T>
+template <typename T, bool HALF>
 __global__ void kb_synth_G(FmgArgs A, int t, int B)
 {
-    const int n = A.lv[t].n;
+    const int n = A.lv[t].n, nh = HALF ? n >> 1 : n;
     const T* psi = static_cast<const T*>(A.psi) + A.psi_off[t];
-    const uint32_t per = static_cast<uint32_t>(A.Ka) * static_cast<uint32_t>(n);
+    const uint32_t per = static_cast<uint32_t>(A.Ka) * static_cast<uint32_t>(nh);
+    const FastDiv by = HALF ? A.lv[t].by_nc : A.lv[t].by_n;
     GRID_STRIDE(idx, B * per)
     {
-        const int i = static_cast<int>(A.lv[t].by_kan.div(idx));
-        const int rem = static_cast<int>(idx - i * per);
-        const int a = static_cast<int>(A.lv[t].by_n.div(rem));
-        const int i2 = rem - a * n;
-        T acc = T(0);
+        const int row = static_cast<int>(by.div(idx));  // sample and group
+        const int i2 = static_cast<int>(idx) - row * nh;
+        const int i = row / A.Ka;
+        const int a = row - i * A.Ka;
+        T acc = T(0), od = T(0);
         const int g1 = A.grp_start[a + 1];
-        if constexpr (sizeof(T) == 4) {
-            // FP32 coefficients sqrt(theta_m) y_m from k_coef32 (the same rounded products)
-            const float* cf = A.c32 + static_cast<size_t>(i) * A.s;
-            for (int g = A.grp_start[a]; g < g1; ++g) acc += cf[A.grp_m[g]] * psi[A.grp_b[g] * n + i2];
-        } else {
-            const double* y = A.Y + static_cast<size_t>(A.samples[i].canon) * A.s;
-            for (int g = A.grp_start[a]; g < g1; ++g) acc += (A.grp_sqrt[g] * y[A.grp_m[g]]) * psi[A.grp_b[g] * n + i2];
+        for (int g = A.grp_start[a]; g < g1; ++g) {
+            const int b = A.grp_b[g];
+            T c;  // FP32: the coefficients of k_coef32 (the same rounded products)
+            if constexpr (sizeof(T) == 4) c = A.c32[static_cast<size_t>(i) * A.s + A.grp_m[g]];
+            else c = A.grp_sqrt[g] * A.Y[static_cast<size_t>(A.samples[i].canon) * A.s + A.grp_m[g]];
+            if (HALF && (b & 1)) od += c * psi[b * n + i2];  // the same branch in every thread of a sample's group
+            else acc += c * psi[b * n + i2];
         }
-        at<T>(A.lv[t].G, i)[rem] = acc;
+        T* G = at<T>(A.lv[t].G, i) + a * n;
+        if constexpr (HALF) {
+            G[i2] = acc + od;
+            G[n - 1 - i2] = acc - od;
+        } else {
+            G[i2] = acc;
+        }
     }
 }
 
@@ -736,22 +752,36 @@ __global__ void k_coef32(FmgArgs A, int B, const double* __restrict__ sq, float*
 }
 
 // k = exp(sum_a psi_a(x1) G_a(x2))
-template <typename T>
+template <typename T, bool HALF>
 __global__ void kb_synth_z(FmgArgs A, int t, int B)
 {
-    const int n = A.lv[t].n;
+    const int n = A.lv[t].n, nh = HALF ? n >> 1 : n;
     const T* psi = static_cast<const T*>(A.psi) + A.psi_off[t];
-    const uint32_t per = static_cast<uint32_t>(n) * static_cast<uint32_t>(n);
+    const uint32_t per = static_cast<uint32_t>(n) * static_cast<uint32_t>(nh);
+    const FastDiv by = HALF ? A.lv[t].by_nc : A.lv[t].by_n, by_n = A.lv[t].by_n;
     GRID_STRIDE(idx, B * per)
     {
-        const int i = static_cast<int>(A.lv[t].by_nn.div(idx));
-        const int p = static_cast<int>(idx - i * per);
-        const int i2 = static_cast<int>(A.lv[t].by_n.div(p));
-        const int i1 = p - i2 * n;
-        const T* G = at<T>(A.lv[t].G, i);
+        const int row = static_cast<int>(by.div(idx));
+        const int i1 = static_cast<int>(idx) - row * nh;
+        const int i = static_cast<int>(by_n.div(row));
+        const int i2 = row - i * n;
+        const T* G = at<T>(A.lv[t].G, i) + i2;
+        T* k = at<T>(A.lv[t].k, i) + i2 * n;
         T z = T(0);
-        for (int a = 0; a < A.Ka; ++a) z += psi[a * n + i1] * G[a * n + i2];
-        at<T>(A.lv[t].k, i)[p] = expT(z);
+        if constexpr (HALF) {
+            T od = T(0);
+            int a = 0;
+            for (; a + 1 < A.Ka; a += 2) {
+                z += psi[a * n + i1] * G[a * n];
+                od += psi[(a + 1) * n + i1] * G[(a + 1) * n];
+            }
+            if (a < A.Ka) z += psi[a * n + i1] * G[a * n];
+            k[i1] = expT(z + od);
+            k[n - 1 - i1] = expT(z - od);
+        } else {
+            for (int a = 0; a < A.Ka; ++a) z += psi[a * n + i1] * G[a * n];
+            k[i1] = expT(z);
+        }
     }
 }
 
@@ -888,7 +918,9 @@ __global__ void kb_gs(FmgArgs A, int t, int B, int colour, int ones)
         const int q = static_cast<int>(idx - i * per);
         const int i2 = static_cast<int>(A.lv[t].by_nc.div(q));
         const Lv<T> L = view<T>(A, t, i);
-        gs_cell(L, ones ? nullptr : L.bc, h2, 2 * (q - i2 * half) + ((i2 + colour) & 1), i2);
+        const int i1 = 2 * (q - i2 * half) + ((i2 + colour) & 1);
+        if (sizeof(T) == 8 && ones) gs_cell<T, true>(L, nullptr, h2, i1, i2);
+        else gs_cell<T, false>(L, ones ? nullptr : L.bc, h2, i1, i2);
     }
 }
 
@@ -1025,6 +1057,7 @@ __global__ void __launch_bounds__(256) kb_rbgs_tile(FmgArgs A, int t, int B, int
 }
 
 // bc of level t-1 = mean over children of (b - A u) on level t.
+// FP64: quad_flux, half the operations of the four children one by one.
 template <typename T>
 __global__ void kb_resid_restrict(FmgArgs A, int t, int B, int ones)
 {
@@ -1062,11 +1095,16 @@ __device__ __forceinline__ void prolong_block(const S* e, int nc, int I1, int I2
         }
     }
     D out[2][2];
+    if constexpr (sizeof(D) == 8) {
+        prolong_quad64(E, out);
+    } else {
 #pragma unroll
-    for (int fy = 0; fy < 2; ++fy)
+        for (int fy = 0; fy < 2; ++fy)
 #pragma unroll
-        for (int fx = 0; fx < 2; ++fx)
-            out[fy][fx] = fma(D(0.5625), E[1][1], fma(D(0.1875), E[1][2 * fx] + E[2 * fy][1], D(0.0625) * E[2 * fy][2 * fx]));
+            for (int fx = 0; fx < 2; ++fx)
+                out[fy][fx] =
+                    fma(D(0.5625), E[1][1], fma(D(0.1875), E[1][2 * fx] + E[2 * fy][1], D(0.0625) * E[2 * fy][2 * fx]));
+    }
     store(out);
 }
 
@@ -1744,7 +1782,7 @@ FmgArgs base_args(mlqmc_ctx* c)
         const LevelPool& P = c->pools[t];
         LevelDesc& d = A.lv[t];
         d.n = c->p.coarse_cells << t;
-        set_divisors(d, c->Ka);
+        set_divisors(d);
         ArrDesc* arr[kPoolArrs] = {&d.u, &d.bc, &d.kx, &d.ky, &d.idiag, &d.k, &d.G, &d.u64, &d.u2};
         for (int a = 0; a < kPoolArrs; ++a) {
             arr[a]->base = P.mem ? P.mem + P.off[a] : nullptr;
@@ -2070,6 +2108,7 @@ mlqmc_status synth_batched(mlqmc_ctx* c, const FmgArgs& A, int t, int B, cudaStr
                                                c->d_sqrt_theta);
     } else if (!uses_tc(c, t) || sizeof(T) != 4) {
         const double M = static_cast<double>(n * n), Ka = c->Ka, sm = c->p.n_modes;
+        const bool half = sizeof(T) == 8 && n >= kHalfFrom;  // n is even
         if constexpr (sizeof(T) == 4) {
             if (!c->c32_ready) {
                 Timed tm(c, kProfSynth, st, work_of<double>(B * 12.0 * sm, B * sm));
@@ -2079,11 +2118,13 @@ mlqmc_status synth_batched(mlqmc_ctx* c, const FmgArgs& A, int t, int B, cudaStr
         }
         {
             Timed tm(c, kProfSynth, st, work_of<T>(B * (sizeof(T) * sm + sizeof(T) * Ka * n), B * 2.0 * sm * n));
-            kb_synth_G<T><<<grid_for(c, B * c->Ka * n), 256, 0, st>>>(A, t, B);
+            if (half) kb_synth_G<T, true><<<grid_for(c, B * c->Ka * (n / 2)), 256, 0, st>>>(A, t, B);
+            else kb_synth_G<T, false><<<grid_for(c, B * c->Ka * n), 256, 0, st>>>(A, t, B);
         }
         {
             Timed tm(c, kProfSynth, st, work_of<T>(B * sizeof(T) * (Ka * n + M), B * 2.0 * Ka * M));
-            kb_synth_z<T><<<grid_for(c, B * n * n), 256, 0, st>>>(A, t, B);
+            if (half) kb_synth_z<T, true><<<grid_for(c, B * n * (n / 2)), 256, 0, st>>>(A, t, B);
+            else kb_synth_z<T, false><<<grid_for(c, B * n * n), 256, 0, st>>>(A, t, B);
         }
     }
     if (part == SynthPart::field) return last_error();
@@ -4040,7 +4081,7 @@ extern "C" mlqmc_status mlqmc_fmg_fields_noalloc(int32_t coarse_cells, int32_t n
     for (int t = 0; t < n_levels; ++t) {
         LevelDesc& d = A.lv[t];
         d.n = coarse_cells << t;
-        set_divisors(d, A.Ka);
+        set_divisors(d);
         ArrDesc* arr[kPoolArrs] = {&d.u, &d.bc, &d.kx, &d.ky, &d.idiag, &d.k, &d.G, &d.u64, &d.u2};
         for (int a = 0; a < kPoolArrs; ++a) {
             arr[a]->base = scratch + offs[t][a];

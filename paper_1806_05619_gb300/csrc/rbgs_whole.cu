@@ -123,12 +123,21 @@ __global__ void __launch_bounds__(WGeom<T, N>::TS * WGeom<T, N>::SPC)
                 }
             }
             T* f = su + (2 * I2) * N + 2 * I1;
+            if constexpr (Gm::F64) {
+                double v[2][2];
+                prolong_quad64(E, v);
 #pragma unroll
-            for (int fy = 0; fy < 2; ++fy)
+                for (int fy = 0; fy < 2; ++fy)
 #pragma unroll
-                for (int fx = 0; fx < 2; ++fx)
-                    f[fy * N + fx] +=
-                        fma(T(0.5625), E[1][1], fma(T(0.1875), E[1][2 * fx] + E[2 * fy][1], T(0.0625) * E[2 * fy][2 * fx]));
+                    for (int fx = 0; fx < 2; ++fx) f[fy * N + fx] += v[fy][fx];
+            } else {
+#pragma unroll
+                for (int fy = 0; fy < 2; ++fy)
+#pragma unroll
+                    for (int fx = 0; fx < 2; ++fx)
+                        f[fy * N + fx] += fma(T(0.5625), E[1][1],
+                                              fma(T(0.1875), E[1][2 * fx] + E[2 * fy][1], T(0.0625) * E[2 * fy][2 * fx]));
+            }
         }
         team_sync<T, N>();
     }
@@ -154,7 +163,13 @@ __global__ void __launch_bounds__(WGeom<T, N>::TS * WGeom<T, N>::SPC)
             const T* kr = skx + y * XP;
             const T w = kr[x], e = kr[x + 1];
             const T nn = sky[c0], so = sky[c0 + N];
-            T acc = h2 * (ones ? T(1) : sb[c0]);
+            T acc;
+            if constexpr (Gm::F64) {
+                acc = h2;  // b = 1: no product (one FP64 operation in six)
+                if (!ones) acc = h2 * sb[c0];
+            } else {
+                acc = h2 * (ones ? T(1) : sb[c0]);
+            }
             acc += w * (x > 0 ? su[c0 - 1] : T(0));
             acc += e * (x < N - 1 ? su[c0 + 1] : T(0));
             acc += nn * (y > 0 ? su[c0 - N] : T(0));
@@ -170,6 +185,14 @@ __global__ void __launch_bounds__(WGeom<T, N>::TS * WGeom<T, N>::SPC)
         T* gbc = at<T>(A.lv[t - 1].bc, ic);
         for (int q = ts; q < NC * NC; q += TS) {
             const int I2 = q / NC, I1 = q - (q / NC) * NC;
+            if constexpr (Gm::F64) {
+                const int o = 2 * I2 * N + 2 * I1;
+                const double qf = quad_flux(skx + 2 * I2 * XP + 2 * I1, sky + o, su + o, N, XP, I1 > 0, I1 < NC - 1,
+                                            I2 > 0, I2 < NC - 1);
+                const double sum = ones ? 4.0 : (sb[o] + sb[o + 1]) + (sb[o + N] + sb[o + N + 1]);
+                gbc[q] = 0.25 * fma(-ih2, qf, sum);
+                continue;
+            }
             T s = T(0);
 #pragma unroll
             for (int d = 0; d < 4; ++d) {
