@@ -210,11 +210,29 @@ constexpr int kTcThreads = 64 + 32 * kEpiWarps;    // TMA warp, MMA warp, epilog
 // of tile i + 1 and the ring never drains between tiles. The ring holds 192 KB
 // of K blocks: four stages of 128 + 256 rows, six of 128 + 128 (one and a half
 // tiles at s = 100).
+//
+// One launch takes several levels, the tiles of one after those of the other:
+// a small call's levels have 1, 2, 8, 32, ... tiles, and one by one each costs
+// a whole pass over K (14 us at s = 1000) that the others' tiles can share:
+// five levels up to 128 x 128, 16 samples, 70 -> 24 us. (Tiles of 32 samples for
+// such calls were measured too: 23.)
+struct LevelTiles {
+    CUtensorMap psi;
+    float* k;
+    size_t stride;  // floats between samples of k
+    int M, B;       // cells, samples
+    int ntiles;     // sample tiles
+    int end;        // tiles of the levels up to this one
+};
+
+struct Levels {
+    CUtensorMap c;
+    LevelTiles lv[mlqmc_kl::kMaxLevels];
+    int count;
+};
+
 template <int NT, bool BF>
-__global__ void __launch_bounds__(kTcThreads, 1) kl_tc_kernel(const __grid_constant__ CUtensorMap tm_psi,
-                                                              const __grid_constant__ CUtensorMap tm_c, int M, int B,
-                                                              int nk, float* __restrict__ kout, size_t kstride,
-                                                              int* err)
+__global__ void __launch_bounds__(kTcThreads, 1) kl_tc_kernel(const __grid_constant__ Levels L, int nk, int* err)
 {
     constexpr int kStages = stages_for<NT>();
     extern __shared__ unsigned char smem_raw[];
@@ -234,8 +252,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) kl_tc_kernel(const __grid_const
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
-    const int ntiles = (B + NT - 1) / NT;
-    const int tiles = ((M + kTileM - 1) / kTileM) * ntiles;  // the Psi map holds whole 128-row tiles (zero rows past M)
+    const int tiles = L.lv[L.count - 1].end;  // the Psi maps hold whole 128-row tiles (zero rows past M)
+    // tile -> its level (l only grows), first cell and first sample
+    auto place = [&](int tile, int& l, int& m0, int& b0) {
+        while (tile >= L.lv[l].end) ++l;
+        const int i = tile - (l > 0 ? L.lv[l - 1].end : 0);
+        m0 = (i / L.lv[l].ntiles) * kTileM;
+        b0 = (i % L.lv[l].ntiles) * NT;
+    };
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
@@ -267,15 +291,17 @@ __global__ void __launch_bounds__(kTcThreads, 1) kl_tc_kernel(const __grid_const
             // producer: K blocks of Psi rows m0.. and C rows b0.. of every tile
             uint32_t g = 0, issued = 0;
             bool ok = true;
+            int l = 0;
             for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
-                const int m0 = (tile / ntiles) * kTileM, b0 = (tile % ntiles) * NT;
+                int m0, b0;
+                place(tile, l, m0, b0);
                 for (int kb = 0; kb < nk; ++kb, ++g) {
                     const uint32_t s = g % kStages;
                     if (g >= kStages && !(ok = wait_or_abort(&empty[s], ((g / kStages) - 1) & 1, abort, err))) break;
                     mbar_expect_tx(&full[s], kABytes + kBBytes);
                     constexpr int kElems = BF ? 64 : kKBlock;  // elements per 128-byte K block
-                    tma_load_2d(sa + s * kABytes, &tm_psi, &full[s], kb * kElems, m0);
-                    tma_load_2d(sb + s * kBBytes, &tm_c, &full[s], kb * kElems, b0);
+                    tma_load_2d(sa + s * kABytes, &L.lv[l].psi, &full[s], kb * kElems, m0);
+                    tma_load_2d(sb + s * kBBytes, &L.c, &full[s], kb * kElems, b0);
                     issued = g + 1;
                 }
             }
@@ -319,14 +345,18 @@ __global__ void __launch_bounds__(kTcThreads, 1) kl_tc_kernel(const __grid_const
         // accumulator columns [h NT / 2, (h + 1) NT / 2), h = (w - 2) / 4
         const int q = warp & 3;
         const int c_lo = ((warp - 2) >> 2) * (NT / 2);
-        int lt = 0;
+        int lt = 0, l = 0;
         for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++lt) {
             const int a = lt & 1;
             // warp-uniform: the TMEM loads below are .sync.aligned
             const bool ready = __all_sync(0xffffffffu, wait_or_abort(&tfull[a], (lt >> 1) & 1, abort, err) ? 1 : 0);
             if (!ready) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const int m0 = (tile / ntiles) * kTileM, b0 = (tile % ntiles) * NT;
+            int m0, b0;
+            place(tile, l, m0, b0);
+            const int M = L.lv[l].M, B = L.lv[l].B;
+            float* __restrict__ kout = L.lv[l].k;
+            const size_t kstride = L.lv[l].stride;
             const int p = m0 + q * 32 + lane;
 #pragma unroll 1
             for (int c = c_lo; c < c_lo + NT / 2; c += 32) {
@@ -574,35 +604,41 @@ bool make_maps(Variant v, const void* d_psi, int M, const void* d_c, int rows_c,
 
 bool prepare_kernel()
 {
-    const int b = static_cast<int>(tc_smem_bytes(kNT)), b128 = static_cast<int>(tc_smem_bytes(128));
-    return cudaFuncSetAttribute(kl_tc_kernel<kNT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, b) ==
-               cudaSuccess &&
-           cudaFuncSetAttribute(kl_tc_kernel<kNT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, b) ==
-               cudaSuccess &&
-           cudaFuncSetAttribute(kl_tc_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, b128) ==
-               cudaSuccess &&
-           cudaFuncSetAttribute(kl_tc_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, b128) ==
-               cudaSuccess;
+    auto set = [](auto* kernel, int nt) {
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    static_cast<int>(tc_smem_bytes(nt))) == cudaSuccess;
+    };
+    return set(kl_tc_kernel<kNT, false>, kNT) && set(kl_tc_kernel<kNT, true>, kNT) && set(kl_tc_kernel<128, false>, 128) &&
+           set(kl_tc_kernel<128, true>, 128);
 }
 
-bool launch(Variant v, const TensorMaps& maps, int M, int B, int s, float* d_k, size_t kstride, int* d_err,
-            cudaStream_t st, int nt)
+bool launch(Variant v, const Field* f, int count, int s, int* d_err, cudaStream_t st, int nt)
 {
-    if (M <= 0 || B <= 0 || (nt != 128 && nt != kNT)) return false;
+    if (count < 1 || count > kMaxLevels || (nt != 128 && nt != kNT)) return false;
     const int nk = static_cast<int>(row_bytes(v, s) / 128);  // 128-byte K blocks
-    CUtensorMap tp, tc;
-    std::memcpy(&tp, maps.psi, sizeof(CUtensorMap));
-    std::memcpy(&tc, nt == 128 ? maps.c128 : maps.c, sizeof(CUtensorMap));
-    const int tiles = ((M + kTileM - 1) / kTileM) * ((B + nt - 1) / nt);
+    Levels L;
+    const TensorMaps& m0 = *f[0].maps;
+    std::memcpy(&L.c, nt == 128 ? m0.c128 : m0.c, sizeof(CUtensorMap));
+    L.count = count;
+    int tiles = 0;
+    for (int i = 0; i < count; ++i) {
+        if (f[i].M <= 0 || f[i].B <= 0) return false;
+        LevelTiles& q = L.lv[i];
+        std::memcpy(&q.psi, f[i].maps->psi, sizeof(CUtensorMap));
+        q.k = f[i].k;
+        q.stride = f[i].stride;
+        q.M = f[i].M;
+        q.B = f[i].B;
+        q.ntiles = (f[i].B + nt - 1) / nt;
+        tiles += ((f[i].M + kTileM - 1) / kTileM) * q.ntiles;
+        q.end = tiles;
+    }
     const int grid = std::min(tiles, sm_count());  // persistent: one CTA per SM
     const size_t smem = tc_smem_bytes(nt);
-    if (nt == 128) {
-        if (v == Variant::TF32) kl_tc_kernel<128, false><<<grid, kTcThreads, smem, st>>>(tp, tc, M, B, nk, d_k, kstride, d_err);
-        else kl_tc_kernel<128, true><<<grid, kTcThreads, smem, st>>>(tp, tc, M, B, nk, d_k, kstride, d_err);
-    } else {
-        if (v == Variant::TF32) kl_tc_kernel<kNT, false><<<grid, kTcThreads, smem, st>>>(tp, tc, M, B, nk, d_k, kstride, d_err);
-        else kl_tc_kernel<kNT, true><<<grid, kTcThreads, smem, st>>>(tp, tc, M, B, nk, d_k, kstride, d_err);
-    }
+    const bool bf = v == Variant::BF16X3;
+    auto go = [&](auto* kernel) { kernel<<<grid, kTcThreads, smem, st>>>(L, nk, d_err); };
+    if (nt == 128) go(bf ? kl_tc_kernel<128, true> : kl_tc_kernel<128, false>);
+    else go(bf ? kl_tc_kernel<kNT, true> : kl_tc_kernel<kNT, false>);
     return cudaGetLastError() == cudaSuccess;
 }
 

@@ -14,6 +14,16 @@ struct alignas(64) TensorMaps {
     unsigned char c128[128];  // the same in boxes of 128 sample rows
 };
 
+constexpr int kMaxLevels = 12;  // levels of one launch (2.4 KB of kernel parameters)
+
+// One level's field: k[b * stride + p] = exp(sum_m Psi[p][m] C[b][m]) for p < M, b < B.
+struct Field {
+    const TensorMaps* maps;
+    int M, B;
+    float* k;
+    size_t stride;
+};
+
 // Operand form: TF32 (one rounding per operand) or split BF16 (three products).
 enum class Variant { TF32, BF16X3 };
 
@@ -36,9 +46,8 @@ bool build_c(Variant v, const double* d_Y, const int* d_canon, int count, int s,
 bool make_maps(Variant v, const void* d_psi, int M, const void* d_c, int rows_c, int s, TensorMaps* maps);
 bool prepare_kernel();
 
-// k[b * kstride + p] = exp(sum_m Psi[p][m] C[b][m]) for p < M (M a multiple of 128), b < B,
-// in tiles of 128 cells x nt samples (nt 128 or 256).
-bool launch(Variant v, const TensorMaps& maps, int M, int B, int s, float* d_k, size_t kstride, int* d_err,
-            cudaStream_t st, int nt = 256);
+// The fields of `count` levels (one context: the same C) in one launch, in
+// tiles of 128 cells x nt samples (nt 128 or 256).
+bool launch(Variant v, const Field* f, int count, int s, int* d_err, cudaStream_t st, int nt = 256);
 
 }  // namespace mlqmc_kl

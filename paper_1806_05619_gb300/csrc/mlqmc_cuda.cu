@@ -857,35 +857,55 @@ __global__ void kb_faces(FmgArgs A, int t, int B)
 // i2, the east boundary face after the last column and the south boundary
 // faces below the last row. The arithmetic of face_x / face_y, operand for
 // operand.
-__global__ void kb_faces4(FmgArgs A, int t, int B)
+__device__ __forceinline__ void faces4(const FmgArgs& A, int t, uint32_t idx)
 {
     const int n = A.lv[t].n;
     const int q = n >> 2;
     const uint32_t per = static_cast<uint32_t>(n) * static_cast<uint32_t>(q);
-    GRID_STRIDE(idx, B * per)
+    const int i = static_cast<int>(A.lv[t].by_nnq.div(idx));
+    const int p4 = static_cast<int>(idx - i * per);
+    const int i2 = static_cast<int>(A.lv[t].by_nq.div(p4));
+    const int i1 = (p4 - i2 * q) * 4;
+    const float* k = at<float>(A.lv[t].k, i);
+    float* kx = at<float>(A.lv[t].kx, i) + i2 * kx_pitch(n);
+    float* ky = at<float>(A.lv[t].ky, i);
+    const float4 c = *reinterpret_cast<const float4*>(k + i2 * n + i1);
+    const float4 fx = make_float4(i1 > 0 ? hmean(k[i2 * n + i1 - 1], c.x) : 2.0f * c.x, hmean(c.x, c.y),
+                                  hmean(c.y, c.z), hmean(c.z, c.w));
+    *reinterpret_cast<float4*>(kx + i1) = fx;
+    if (i1 + 4 == n) kx[n] = 2.0f * c.w;
+    float4 fy;
+    if (i2 > 0) {
+        const float4 a = *reinterpret_cast<const float4*>(k + (i2 - 1) * n + i1);
+        fy = make_float4(hmean(a.x, c.x), hmean(a.y, c.y), hmean(a.z, c.z), hmean(a.w, c.w));
+    } else {
+        fy = make_float4(2.0f * c.x, 2.0f * c.y, 2.0f * c.z, 2.0f * c.w);
+    }
+    *reinterpret_cast<float4*>(ky + i2 * n + i1) = fy;
+    if (i2 == n - 1)
+        *reinterpret_cast<float4*>(ky + n * n + i1) = make_float4(2.0f * c.x, 2.0f * c.y, 2.0f * c.z, 2.0f * c.w);
+}
+
+__global__ void kb_faces4(FmgArgs A, int t, int B)
+{
+    const int n = A.lv[t].n;
+    GRID_STRIDE(idx, B * (static_cast<uint32_t>(n) * static_cast<uint32_t>(n >> 2))) faces4(A, t, idx);
+}
+
+// The faces of all levels of a small call in one launch: end[l] = quads of the
+// levels up to l (levels below 2^31 quads together).
+struct FaceLevels {
+    uint32_t end[MLQMC_MAX_LEVELS];
+    int count;
+};
+
+__global__ void kb_faces4_levels(FmgArgs A, FaceLevels L)
+{
+    int t = 0;
+    GRID_STRIDE(idx, L.end[L.count - 1])
     {
-        const int i = static_cast<int>(A.lv[t].by_nnq.div(idx));
-        const int p4 = static_cast<int>(idx - i * per);
-        const int i2 = static_cast<int>(A.lv[t].by_nq.div(p4));
-        const int i1 = (p4 - i2 * q) * 4;
-        const float* k = at<float>(A.lv[t].k, i);
-        float* kx = at<float>(A.lv[t].kx, i) + i2 * kx_pitch(n);
-        float* ky = at<float>(A.lv[t].ky, i);
-        const float4 c = *reinterpret_cast<const float4*>(k + i2 * n + i1);
-        const float4 fx = make_float4(i1 > 0 ? hmean(k[i2 * n + i1 - 1], c.x) : 2.0f * c.x, hmean(c.x, c.y),
-                                      hmean(c.y, c.z), hmean(c.z, c.w));
-        *reinterpret_cast<float4*>(kx + i1) = fx;
-        if (i1 + 4 == n) kx[n] = 2.0f * c.w;
-        float4 fy;
-        if (i2 > 0) {
-            const float4 a = *reinterpret_cast<const float4*>(k + (i2 - 1) * n + i1);
-            fy = make_float4(hmean(a.x, c.x), hmean(a.y, c.y), hmean(a.z, c.z), hmean(a.w, c.w));
-        } else {
-            fy = make_float4(2.0f * c.x, 2.0f * c.y, 2.0f * c.z, 2.0f * c.w);
-        }
-        *reinterpret_cast<float4*>(ky + i2 * n + i1) = fy;
-        if (i2 == n - 1)
-            *reinterpret_cast<float4*>(ky + n * n + i1) = make_float4(2.0f * c.x, 2.0f * c.y, 2.0f * c.z, 2.0f * c.w);
+        while (idx >= L.end[t]) ++t;  // idx only grows
+        faces4(A, t, idx - (t > 0 ? L.end[t - 1] : 0u));
     }
 }
 
@@ -2070,12 +2090,12 @@ bool uses_tc(const mlqmc_ctx* c, int t)
     return c->kl_tc && c->d_psi_tc[t] != nullptr;
 }
 
-enum class SynthPart { all, field, faces };
+enum class SynthPart { all, field, faces, idiag };
 
 // Batched KL field and faces of level t for samples 0..B-1. The field comes
 // from the tensor-core contraction (mixed forms, every level)
 // or from the separable SIMT sum; the C operand must already be built.
-// part: the tensor-core field alone, or the faces alone (after it).
+// part: the tensor-core field alone, the faces and 1/D alone (after it), or 1/D alone.
 template <typename T>
 mlqmc_status synth_batched(mlqmc_ctx* c, const FmgArgs& A, int t, int B, cudaStream_t st,
                            SynthPart part = SynthPart::all)
@@ -2083,7 +2103,7 @@ mlqmc_status synth_batched(mlqmc_ctx* c, const FmgArgs& A, int t, int B, cudaStr
     LevelTag lt(c, t);
     const int64_t n = c->p.coarse_cells << t;
     if constexpr (sizeof(T) == 4) {
-        if (uses_tc(c, t) && part != SynthPart::faces) {
+        if (uses_tc(c, t) && (part == SynthPart::all || part == SynthPart::field)) {
             const LevelPool& P = c->pools[t];
             float* k = reinterpret_cast<float*>(P.mem + P.off[kK]);
             const double M = static_cast<double>(n * n);
@@ -2092,12 +2112,12 @@ mlqmc_status synth_batched(mlqmc_ctx* c, const FmgArgs& A, int t, int B, cudaStr
             w.bytes = 4.0 * (M * B + M * K + B * K);  // k out, Psi and C in
             w.ftc = 2.0 * M * c->p.n_modes * B;
             Timed tm(c, kProfKlTc, st, w);
-            if (!mlqmc_kl::launch(c->kl_variant, c->kl_maps[t], static_cast<int>(n * n), B, c->p.n_modes, k,
-                                  P.stride[kK] / sizeof(float), c->d_status, st, kl_nt_for(c, t, B)))
+            const mlqmc_kl::Field f{&c->kl_maps[t], static_cast<int>(n * n), B, k, P.stride[kK] / sizeof(float)};
+            if (!mlqmc_kl::launch(c->kl_variant, &f, 1, c->p.n_modes, c->d_status, st, kl_nt_for(c, t, B)))
                 return MLQMC_ERR_CUDA;
         }
     }
-    if (part == SynthPart::faces) {
+    if (part == SynthPart::faces || part == SynthPart::idiag) {
     } else if (c->matern && (!uses_tc(c, t) || sizeof(T) != 4)) {
         const double M = static_cast<double>(n * n), sm = c->p.n_modes;
         Timed tm(c, kProfSynth, st,
@@ -2129,7 +2149,7 @@ mlqmc_status synth_batched(mlqmc_ctx* c, const FmgArgs& A, int t, int B, cudaStr
     }
     if (part == SynthPart::field) return last_error();
     const double es = sizeof(T), Mc = cells_of(c, t), Fc = faces_of(c, t);
-    {
+    if (part != SynthPart::idiag) {
         Timed tm(c, kProfSynth, st, work_of<T>(B * es * (Mc + 2.0 * Fc), B * 6.0 * Fc));
         if (sizeof(T) == 4 && n % 4 == 0) kb_faces4<<<grid_for(c, B * n * n / 4), 256, 0, st>>>(A, t, B);
         else kb_faces<T><<<grid_for(c, B * n * n), 256, 0, st>>>(A, t, B);
@@ -2139,6 +2159,58 @@ mlqmc_status synth_batched(mlqmc_ctx* c, const FmgArgs& A, int t, int B, cudaStr
         kb_idiag<T><<<grid_for(c, B * n * n), 256, 0, st>>>(A, t, B);
     }
     return last_error();
+}
+
+// Fields of all levels up to Lmax from the tensor cores: one launch per tile
+// width (level by level while the profile attributes time to levels).
+mlqmc_status fields_tc(mlqmc_ctx* c, const FmgArgs& A, const int* Bt, int Lmax, cudaStream_t st)
+{
+    static_assert(mlqmc_kl::kMaxLevels >= MLQMC_MAX_LEVELS, "levels of one launch");
+    if (c->profiling) {
+        mlqmc_status s = MLQMC_OK;
+        for (int t = 0; s == MLQMC_OK && t <= Lmax && Bt[t] > 0; ++t)
+            s = synth_batched<float>(c, A, t, Bt[t], st, SynthPart::field);
+        return s;
+    }
+    for (const int nt : {256, 128}) {
+        mlqmc_kl::Field f[MLQMC_MAX_LEVELS];
+        int count = 0;
+        for (int t = Lmax; t >= 0; --t) {  // the largest level first: the small ones fill the last wave
+            if (Bt[t] <= 0 || kl_nt_for(c, t, Bt[t]) != nt) continue;
+            const LevelPool& P = c->pools[t];
+            const int n = c->p.coarse_cells << t;
+            f[count++] = {&c->kl_maps[t], n * n, Bt[t], reinterpret_cast<float*>(P.mem + P.off[kK]),
+                          P.stride[kK] / sizeof(float)};
+        }
+        if (count == 0) continue;
+        Timed tm(c, kProfKlTc, st);
+        if (!mlqmc_kl::launch(c->kl_variant, f, count, c->p.n_modes, c->d_status, st, nt)) return MLQMC_ERR_CUDA;
+    }
+    return MLQMC_OK;
+}
+
+// Cells of a call's levels together up to which one launch forms all faces:
+// below it a launch per level costs its latency (2 us and the gap before the
+// next), above it level 0's factorisation should not wait for the large levels' faces.
+constexpr int64_t kFacesTogether = int64_t{1} << 22;
+
+// Faces of levels 0..Lmax in one launch; false when the call is not of that kind.
+bool faces_together(mlqmc_ctx* c, const FmgArgs& A, const int* Bt, int Lmax, cudaStream_t st)
+{
+    if (c->profiling || c->p.coarse_cells % 4 != 0) return false;
+    FaceLevels L{};
+    int64_t quads = 0;
+    for (int t = 0; t <= Lmax && Bt[t] > 0; ++t) {
+        const int64_t n = c->p.coarse_cells << t;
+        quads += Bt[t] * n * (n / 4);
+        if (4 * quads > kFacesTogether) return false;
+        L.end[t] = static_cast<uint32_t>(quads);
+        L.count = t + 1;
+    }
+    if (L.count == 0) return false;
+    Timed tm(c, kProfSynth, st);
+    kb_faces4_levels<<<grid_for(c, quads), 256, 0, st>>>(A, L);
+    return true;
 }
 
 // C operand of the tensor-core contraction for samples 0..count-1 (normals in rank order).
@@ -2920,10 +2992,10 @@ mlqmc_status tune_kl(mlqmc_ctx* c)
         for (int cls = 0; cls < 2 && res == MLQMC_OK; ++cls) {
             for (int k = 0; k < 2 && res == MLQMC_OK; ++k) {
                 float ms = 0.0f, tot = 0.0f;
+                const mlqmc_kl::Field f{&c->kl_maps[t], M, Bs[cls], out, static_cast<size_t>(M)};
                 for (int rep = 0; rep < 4 && res == MLQMC_OK; ++rep) {  // one untimed launch, then three timed
                     if (!ok(cudaEventRecord(e0, st)) ||
-                        !mlqmc_kl::launch(c->kl_variant, c->kl_maps[t], M, Bs[cls], c->p.n_modes, out,
-                                          static_cast<size_t>(M), c->d_status, st, NTs[k]) ||
+                        !mlqmc_kl::launch(c->kl_variant, &f, 1, c->p.n_modes, c->d_status, st, NTs[k]) ||
                         !ok(cudaEventRecord(e1, st)) || !ok(cudaEventSynchronize(e1)) ||
                         !ok(cudaEventElapsedTime(&ms, e0, e1)))
                         res = MLQMC_ERR_CUDA;
@@ -3000,21 +3072,24 @@ mlqmc_status run_chunk(mlqmc_ctx* c, int count, const int* Bt, int Lmax, double*
         c->c32_ready = false;
         return MLQMC_ERR_CUDA;
     }
-    s = is_mixed(p) ? synth_batched<float>(c, A, 0, Bt[0], c->side) : synth_batched<double>(c, A, 0, Bt[0], c->side);
     if (is_mixed(p) && all_tc) {
         // the persistent contractions cannot start beside the factorisation's
         // CTAs (both need most of an SM's shared memory): the main stream
-        // issues the other levels' contractions first, the factorisation
-        // follows them and runs beside those levels' faces
-        for (int t = 1; s == MLQMC_OK && t <= Lmax && Bt[t] > 0; ++t)
-            s = synth_batched<float>(c, A, t, Bt[t], st, SynthPart::field);
+        // forms every level's field first, level 0's faces and factorisation
+        // follow on the side stream, beside the other levels' faces
+        // (a small call: all levels' faces in one launch before the fork)
+        s = fields_tc(c, A, Bt, Lmax, st);
+        const bool together = s == MLQMC_OK && faces_together(c, A, Bt, Lmax, st);
+        const SynthPart rest = together ? SynthPart::idiag : SynthPart::faces;
         if (!ok(cudaEventRecord(c->ev_fields, st)) || !ok(cudaStreamWaitEvent(c->side, c->ev_fields, 0)))
             s = MLQMC_ERR_CUDA;
+        if (s == MLQMC_OK) s = synth_batched<float>(c, A, 0, Bt[0], c->side, rest);
         if (s == MLQMC_OK) s = launch_level0(c, A, Bt[0], c->side);
         if (!ok(cudaEventRecord(c->ev_join, c->side))) s = MLQMC_ERR_CUDA;
         for (int t = 1; s == MLQMC_OK && t <= Lmax && Bt[t] > 0; ++t)
-            s = synth_batched<float>(c, A, t, Bt[t], st, SynthPart::faces);
+            s = synth_batched<float>(c, A, t, Bt[t], st, rest);
     } else {
+        s = is_mixed(p) ? synth_batched<float>(c, A, 0, Bt[0], c->side) : synth_batched<double>(c, A, 0, Bt[0], c->side);
         if (s == MLQMC_OK) s = launch_level0(c, A, Bt[0], c->side);
         if (!ok(cudaEventRecord(c->ev_join, c->side))) s = MLQMC_ERR_CUDA;
         for (int t = 1; s == MLQMC_OK && t <= Lmax && Bt[t] > 0; ++t)
