@@ -25,6 +25,8 @@
 
 #include "fmg_device.cuh"
 #include "fmg_small.h"
+#include "level0_lanes.cuh"
+#include "level0_pairs.h"
 #include "mlqmc_internal.h"
 #include "rbgs_stream.h"
 #include "rbgs_tma.h"
@@ -185,24 +187,6 @@ __global__ void k_points_mixed(const SampleDesc* __restrict__ smp, int count, in
 // at fac[(r*(n0+1) + d) * stride + i] (coalesced across samples); the
 // diagonal d = 0 holds 1/L(r, r).
 // ---------------------------------------------------------------------------
-template <typename T>
-__device__ __forceinline__ T band_a(const T* kx, const T* ky, int n0, int r, int l)
-{
-    const int r1 = r % n0, r2 = r / n0;
-    if (l == 1 && r1 > 0) return -kx[r2 * kx_pitch(n0) + r1];
-    if (l == n0) return -ky[r2 * n0 + r1];
-    return T(0);
-}
-
-// Diagonal of row j of h0^2 A_0: the sum of the cell's four faces.
-template <typename T>
-__device__ __forceinline__ double level0_diag(const T* kx, const T* ky, int n0, int j)
-{
-    const int j1 = j % n0, j2 = j / n0;
-    return widen(kx[j2 * kx_pitch(n0) + j1]) + widen(kx[j2 * kx_pitch(n0) + j1 + 1]) + widen(ky[j2 * n0 + j1]) +
-           widen(ky[(j2 + 1) * n0 + j1]);
-}
-
 // Factor, exact FP64 solve with f = 1, F_0; the mixed forms also keep an FP32
 // copy of the factor for the coarse solves of their FP32 V-cycles.
 template <typename T, bool MX>
@@ -323,7 +307,7 @@ __device__ __forceinline__ double tree16(double (&s)[16])
 // with the last NC values in registers); shared memory holds the ring only,
 // so that all samples of a call fit on the GPU at once. Every sum takes its
 // oldest term first, the order in which kb_level0_lanes' updates arrive.
-template <typename T, bool MX, int NC>
+template <int NC>
 __global__ void __launch_bounds__(64) kb_level0_fixed(FmgArgs A, int B)
 {
     constexpr int N = NC * NC, W = NC + 1, TPB = 64;
@@ -332,14 +316,13 @@ __global__ void __launch_bounds__(64) kb_level0_fixed(FmgArgs A, int B)
     const int tid = threadIdx.x;
     const size_t cs = A.chol.stride;
     double* fac = reinterpret_cast<double*>(A.chol.base);
-    float* f32 = reinterpret_cast<float*>(A.chol32);
     const double h2 = 1.0 / (static_cast<double>(NC) * NC);
     for (int base = blockIdx.x * TPB; base < B; base += gridDim.x * TPB) {
         const int i = base + tid;
         if (i >= B) continue;  // no barriers in this kernel: shared rows are private to the thread
         auto Rs = [&](int slot, int e) -> double& { return ring[(slot * W + e) * TPB + tid]; };
-        const Lv<T> L0 = view<T>(A, 0, i);
-        double* x = (MX || A.refine) ? L0.u64 : reinterpret_cast<double*>(L0.u);
+        const Lv<double> L0 = view<double>(A, 0, i);
+        double* x = A.refine ? L0.u64 : L0.u;
         double win[NC];  // win[q - 1] = y_(j - q), the forward values of the last NC rows
 #pragma unroll
         for (int q = 0; q < NC; ++q) win[q] = 0.0;
@@ -370,7 +353,6 @@ __global__ void __launch_bounds__(64) kb_level0_fixed(FmgArgs A, int B)
             for (int e = 0; e <= NC; ++e) {
                 if (!FULL && e > j) break;
                 fac[static_cast<size_t>(j * W + e) * cs + i] = Rs(s0, e);
-                if constexpr (MX) f32[static_cast<size_t>(j * W + e) * cs + i] = narrow(Rs(s0, e));
             }
 #pragma unroll
             for (int l = 1; l <= NC; ++l) {
@@ -404,7 +386,6 @@ __global__ void __launch_bounds__(64) kb_level0_fixed(FmgArgs A, int B)
 #pragma unroll
             for (int q = NC - 1; q > 0; --q) win[q] = win[q - 1];
             win[0] = xr;
-            if constexpr (MX) reinterpret_cast<float*>(L0.u)[r] = narrow(xr);  // FP32 copy for the first FMG interpolation
         }
         double F0;
         if (A.qoi == MLQMC_QOI_MEAN) {
@@ -424,191 +405,11 @@ __global__ void __launch_bounds__(64) kb_level0_fixed(FmgArgs A, int B)
     }
 }
 
-// Level 0 for n0 = NC on several lanes per sample (LPR lanes for each of the
-// NC rows of the working window, NC LPR lanes in all). On GB300 an FP64 warp
-// instruction holds its SM sub-partition for about 70 cycles whatever its
-// active lanes, so what a sample costs is its FP64 warp instructions, and one
-// thread's ~4,700 of them take 0.2 ms however few samples a call has. Here
-// column j updates the whole trailing window at once (right-looking): lane
-// (p, g) keeps row r = p mod NC and its columns c = g mod LPR in registers
-// (register c mod NC), the diagonal and the right-hand side ride along, and a
-// column costs its reciprocal square root (5), one scaling and NC/LPR + 1 (or
-// + 3, LPR = 1) updates. Registers whose column is already eliminated take
-// part with stale values and are reset when their row is replaced; the
-// finished column goes to shared memory (backward substitution, pushed the
-// same way) and to the global factor. Sums take their oldest term first, as
-// in kb_level0_fixed: the same bits.
+// FP64 form of n0 = 4, 6, 8, 10: several lanes per sample, a warp for SPW samples.
 template <int NC, int LPR>
-struct L0Geom {
-    static constexpr int TL = NC * LPR;      // lanes that work on a sample
-    static constexpr int SEG = TL <= 4 ? 4 : (TL <= 8 ? 8 : (TL <= 16 ? 16 : 32));  // lanes that a sample occupies
-    static constexpr int SPW = 32 / SEG;     // samples per warp
-    static constexpr int N = NC * NC;
-    static constexpr int oL = 0;             // column j of L below the diagonal: [j * NC + row mod NC]
-    static constexpr int oR = oL + N * NC;   // 1 / L(j, j)
-    static constexpr int oY = oR + N;        // forward values, then the solution
-    static constexpr int oD = oY + N;        // diagonal sums of h0^2 A_0
-    static constexpr int oA = oD + N;        // -L.kx: coupling of row r to r - 1, then of row r to r - NC
-    static constexpr int per = oA + 2 * N;   // doubles per sample
-    static constexpr size_t bytes = sizeof(double) * per * SPW;
-};
-
-template <typename T, bool MX, int NC, int LPR>
 __global__ void __launch_bounds__(32) kb_level0_lanes(FmgArgs A, int B)
 {
-    using Gm = L0Geom<NC, LPR>;
-    constexpr int N = NC * NC, W = NC + 1, KR = (NC + LPR - 1) / LPR;
-    static_assert(LPR == 1 || LPR == 4, "the diagonal and the right-hand side take two groups, the column a third");
-    extern __shared__ double l0sh[];
-    const int lane = threadIdx.x, team = lane / Gm::SEG, tl = lane - team * Gm::SEG;
-    const int i = blockIdx.x * Gm::SPW + team;
-    const bool live = i < B;
-    const int si = live ? i : B - 1;  // lanes past B compute on sample B-1 and store nothing
-    const bool work = tl < Gm::TL;    // NC = 6: lanes past the window stay idle but converged
-    const int p = work ? tl / LPR : 0, g = work ? tl - p * LPR : 0;
-    const int t0 = team * Gm::SEG;
-    double* S = l0sh + static_cast<size_t>(team) * Gm::per;
-    const size_t cs = A.chol.stride;
-    double* fac = reinterpret_cast<double*>(A.chol.base);
-    float* f32 = reinterpret_cast<float*>(A.chol32);
-    const double h2 = 1.0 / (static_cast<double>(NC) * NC);
-    const Lv<T> L0 = view<T>(A, 0, si);
-    for (int r = tl; r < N; r += Gm::SEG) {
-        S[Gm::oD + r] = level0_diag(L0.kx, L0.ky, NC, r);
-        S[Gm::oA + 2 * r] = widen(band_a(L0.kx, L0.ky, NC, r, 1));
-        S[Gm::oA + 2 * r + 1] = r >= NC ? widen(band_a(L0.kx, L0.ky, NC, r, NC)) : 0.0;
-    }
-    __syncwarp();
-    // LPR = 4: group (p + 2) mod 4 of row slot p holds its diagonal, group (p + 1) mod 4 its
-    // right-hand side: never the group of the column being eliminated when the slot is the pivot
-    const int gd = LPR == 1 ? 0 : (p + 2) % LPR;
-    double off[KR];  // column c of the lane's row, c mod NC = g + LPR k
-    double X, V = 0.0;  // diagonal or right-hand side (LPR = 1: diagonal and right-hand side)
-    auto reset = [&](int r) {  // row r enters the window
-        const bool in = r < N;
-        const int rr = in ? r : 0;
-#pragma unroll
-        for (int k = 0; k < KR; ++k) {
-            const int cm = g + LPR * k;
-            double a = 0.0;
-            if (cm == (r + NC - 1) % NC) a = S[Gm::oA + 2 * rr];
-            if (cm == r % NC) a = S[Gm::oA + 2 * rr + 1];
-            off[k] = in ? a : 0.0;
-        }
-        const double d = S[Gm::oD + rr];
-        if constexpr (LPR == 1) {
-            X = d;
-            V = h2;
-        } else {
-            X = g == gd ? d : h2;
-        }
-    };
-    reset(p);
-    for (int j0 = 0; j0 < N; j0 += NC) {
-#pragma unroll
-        for (int sj = 0; sj < NC; ++sj) {
-            const int j = j0 + sj;
-            constexpr int L1 = LPR - 1;
-            const int gc = sj & L1, kc = sj / LPR;        // group and register of the column being eliminated
-            const int ld = LPR == 1 ? 0 : (sj + 2) % LPR, lv = LPR == 1 ? 0 : (sj + 1) % LPR;
-            const double d = __shfl_sync(0xffffffffu, X, t0 + sj * LPR + ld);
-            const double rl = rsqrt64(d);
-            double yj;
-            double Lm;
-            if constexpr (LPR == 1) {
-                const double vj = __shfl_sync(0xffffffffu, V, t0 + sj);
-                if (p == sj) reset(j + NC);
-                Lm = off[kc] * rl;
-                yj = vj * rl;
-            } else {
-                const double xo = X;
-                if (p == sj) reset(j + NC);
-                Lm = ((p == sj && g == lv) ? xo : off[kc]) * rl;  // one multiplication: column j and y_j
-                yj = __shfl_sync(0xffffffffu, Lm, t0 + sj * LPR + lv);
-            }
-            const double Lr = LPR == 1 ? Lm : __shfl_sync(0xffffffffu, Lm, t0 + p * LPR + gc);
-#pragma unroll
-            for (int k = 0; k < KR; ++k) {
-                const int cm = g + LPR * k;  // row slot of column c
-                if (LPR == 1 && cm == sj) continue;
-                const double Lc = __shfl_sync(0xffffffffu, Lm, t0 + (cm < NC ? cm : 0) * LPR + gc);
-                if (cm != sj) off[k] = fma(-Lr, Lc, off[k]);
-            }
-            if constexpr (LPR == 1) {
-                X = fma(-Lr, Lr, X);
-                V = fma(-Lr, yj, V);
-            } else {
-                X = fma(-Lr, g == gd ? Lr : yj, X);
-            }
-            if (work && g == gc) S[Gm::oL + j * NC + p] = Lr;
-            if (tl == 0) {
-                S[Gm::oR + j] = rl;
-                S[Gm::oY + j] = yj;
-            }
-        }
-    }
-    __syncwarp();
-    // the factor to global memory in one pass (inside the loop its address
-    // arithmetic and, mixed forms, the rounding to FP32 sat on the critical path)
-    if (live) {
-        auto put = [&](int q, double v) {
-            if constexpr (MX) f32[static_cast<size_t>(q) * cs + i] = narrow(v);
-            else fac[static_cast<size_t>(q) * cs + i] = v;
-        };
-        for (int q = tl; q < N * NC; q += Gm::SEG) {  // column j, row slot q mod NC: row j + l
-            const int j = q / NC, l = (q - j * NC + NC - j % NC) % NC;
-            const int lr = l ? l : NC;
-            if (j + lr < N) put((j + lr) * W + lr, S[Gm::oL + q]);
-        }
-        for (int j = tl; j < N; j += Gm::SEG) put(j * W, S[Gm::oR + j]);
-    }
-    __syncwarp();
-    // backward substitution: lane p < NC (LPR lanes of a slot alike) keeps the
-    // pending value of the row of slot p; row r's solution updates rows r-1..r-NC
-    double v = S[Gm::oY + N - NC + p];
-    for (int r0 = N - NC; r0 >= 0; r0 -= NC) {
-#pragma unroll
-        for (int sr = NC - 1; sr >= 0; --sr) {
-            const int r = r0 + sr;
-            const int c = p < sr ? r0 + p : r0 + p - NC;  // the slot's row below r (slot sr: row r - NC enters)
-            const double Lc = c >= 0 ? S[Gm::oL + c * NC + sr] : 0.0;
-            const double xr = __shfl_sync(0xffffffffu, v, t0 + sr * LPR) * S[Gm::oR + r];
-            if (p == sr) v = c >= 0 ? S[Gm::oY + c] : 0.0;
-            v = fma(-Lc, xr, v);
-            if (tl == 0) S[Gm::oY + r] = xr;
-        }
-    }
-    __syncwarp();
-    double* x = (MX || A.refine) ? L0.u64 : reinterpret_cast<double*>(L0.u);
-    if (live)
-        for (int r = tl; r < N; r += Gm::SEG) {
-            x[r] = S[Gm::oY + r];
-            if constexpr (MX) reinterpret_cast<float*>(L0.u)[r] = narrow(S[Gm::oY + r]);  // FP32 copy for the first FMG interpolation
-        }
-    double F0;
-    if (A.qoi == MLQMC_QOI_MEAN) {
-        constexpr int Q = Gm::SEG >= 16 ? 1 : 16 / Gm::SEG;  // partial sums per lane: c = tl + SEG q
-        double s[Q];
-#pragma unroll
-        for (int q = 0; q < Q; ++q) {
-            const int c = (tl & 15) + Gm::SEG * q;
-            s[q] = S[Gm::oY + c];
-            for (int r = 16 + c; r < N; r += 16) s[q] += S[Gm::oY + r];
-        }
-#pragma unroll
-        for (int w = Q / 2; w > 0; w >>= 1)
-#pragma unroll
-            for (int q = 0; q < w; ++q) s[q] += s[q + w];
-        double acc = s[0];
-#pragma unroll
-        for (int w = Gm::SEG >= 16 ? 8 : Gm::SEG / 2; w > 0; w >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, w);
-        F0 = acc / static_cast<double>(N);
-    } else {
-        constexpr int m = NC / 2;
-        const double* y = S + Gm::oY;
-        F0 = 0.25 * (y[(m - 1) * NC + (m - 1)] + y[(m - 1) * NC + m] + y[m * NC + (m - 1)] + y[m * NC + m]);
-    }
-    if (live && tl == 0) A.F[static_cast<size_t>(i) * A.n_levels] = F0;
+    level0_warp<double, false, NC, LPR>(A, B, blockIdx.x * L0Geom<NC, LPR>::SPW, 0xffffffffu);
 }
 
 template <int NC>
@@ -1963,11 +1764,11 @@ int level0_lanes(int n0, int B)
     return B < kLevel0FourLanes && 4 * n0 <= 32 ? 4 : 1;
 }
 
-template <typename T, bool MX, int NC, int LPR>
+template <int NC, int LPR>
 void launch_lanes(const FmgArgs& A, int B, cudaStream_t st)
 {
     using Gm = L0Geom<NC, LPR>;
-    kb_level0_lanes<T, MX, NC, LPR><<<(B + Gm::SPW - 1) / Gm::SPW, 32, Gm::bytes, st>>>(A, B);
+    kb_level0_lanes<NC, LPR><<<(B + Gm::SPW - 1) / Gm::SPW, 32, Gm::bytes, st>>>(A, B);
 }
 
 // Level-0 factor, exact solve and F_0 of samples 0..B-1.
@@ -1982,29 +1783,29 @@ mlqmc_status launch_level0(mlqmc_ctx* c, const FmgArgs& A, int B, cudaStream_t s
                    (8.0 + es) * N0 + 8.0);
     w.f64 = B * (N0 * n0 * n0 + 4.0 * N0 * n0);
     Timed tm(c, kProfSmall, st, w);
+    const int n0c = c->p.coarse_cells;
+    if (is_mixed(c->p)) {
+        if (mlqmc_level0::supported(n0c)) return mlqmc_level0::launch(A, n0c, B, st) ? MLQMC_OK : MLQMC_ERR_CUDA;
+        kb_level0<float, true><<<grid_for(c, B, 128), 128, 0, st>>>(A, B);
+        return last_error();
+    }
     // n0 = 8: one wave of resident CTAs (shared memory allows five per SM),
     // each looping over its samples, so that all of them are placed at once
     // and the other stream's kernels are not queued behind a second wave
     int per_sm = 8;
-    if (c->p.coarse_cells == 8) {
-        const bool mx = is_mixed(c->p);
-        if (!ok(mx ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kb_level0_fixed<float, true, 8>, 64,
-                                                                  level0_smem<8>())
-                   : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kb_level0_fixed<double, false, 8>, 64,
-                                                                  level0_smem<8>())))
+    if (n0c == 8) {
+        if (!ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kb_level0_fixed<8>, 64, level0_smem<8>())))
             return MLQMC_ERR_CUDA;
         per_sm = std::max(1, per_sm);
     }
     const int g64 = std::max(1, std::min((B + 63) / 64, c->sm_count * per_sm));
-    const int n0c = c->p.coarse_cells;
     const int lanes = level0_lanes(n0c, B);
-    const bool mx = is_mixed(c->p);
     auto by_lanes = [&](auto nc) {
         constexpr int NC = decltype(nc)::value;
         if constexpr (NC * 4 <= 32) {
-            if (lanes == 4) return mx ? launch_lanes<float, true, NC, 4>(A, B, st) : launch_lanes<double, false, NC, 4>(A, B, st);
+            if (lanes == 4) return launch_lanes<NC, 4>(A, B, st);
         }
-        mx ? launch_lanes<float, true, NC, 1>(A, B, st) : launch_lanes<double, false, NC, 1>(A, B, st);
+        launch_lanes<NC, 1>(A, B, st);
     };
     if (lanes && n0c == 8) {
         by_lanes(std::integral_constant<int, 8>());
@@ -2014,14 +1815,10 @@ mlqmc_status launch_level0(mlqmc_ctx* c, const FmgArgs& A, int B, cudaStream_t s
         by_lanes(std::integral_constant<int, 6>());
     } else if (lanes && n0c == 10) {
         by_lanes(std::integral_constant<int, 10>());
-    } else if (c->p.coarse_cells == 8) {
-        if (is_mixed(c->p)) kb_level0_fixed<float, true, 8><<<g64, 64, level0_smem<8>(), st>>>(A, B);
-        else kb_level0_fixed<double, false, 8><<<g64, 64, level0_smem<8>(), st>>>(A, B);
-    } else if (c->p.coarse_cells == 4) {
-        if (is_mixed(c->p)) kb_level0_fixed<float, true, 4><<<g64, 64, level0_smem<4>(), st>>>(A, B);
-        else kb_level0_fixed<double, false, 4><<<g64, 64, level0_smem<4>(), st>>>(A, B);
-    } else if (is_mixed(c->p)) {
-        kb_level0<float, true><<<grid_for(c, B, 128), 128, 0, st>>>(A, B);
+    } else if (n0c == 8) {
+        kb_level0_fixed<8><<<g64, 64, level0_smem<8>(), st>>>(A, B);
+    } else if (n0c == 4) {
+        kb_level0_fixed<4><<<g64, 64, level0_smem<4>(), st>>>(A, B);
     } else {
         kb_level0<double, false><<<grid_for(c, B, 128), 128, 0, st>>>(A, B);
     }
@@ -3407,9 +3204,7 @@ extern "C" mlqmc_status mlqmc_create(const mlqmc_problem* p, int64_t max_samples
 
     // shared memory of the tiled smoother
     if (!(tile_attrs<32>() && tile_attrs<16>() && tile_attrs<8>() && mlqmc_stream::prepare() &&
-          ok(cudaFuncSetAttribute(kb_level0_fixed<float, true, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  static_cast<int>(level0_smem<8>()))) &&
-          ok(cudaFuncSetAttribute(kb_level0_fixed<double, false, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+          ok(cudaFuncSetAttribute(kb_level0_fixed<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   static_cast<int>(level0_smem<8>()))))) {
         free_ctx(c);
         return MLQMC_ERR_CUDA;
@@ -3645,7 +3440,7 @@ mlqmc_status round_graph(mlqmc_ctx* c, int count, const int* Bt, int Lmax, doubl
         key.push_back(Bt[t] > 0 ? smoother_for(c, t, Bt[t]) : -1);
         key.push_back(Bt[t] > 0 ? kl_nt_for(c, t, Bt[t]) : 0);
     }
-    key.push_back(level0_lanes(c->p.coarse_cells, Bt[0]));
+    key.push_back(is_mixed(c->p) ? mlqmc_level0::four_lanes(c->p.coarse_cells, Bt[0]) : level0_lanes(c->p.coarse_cells, Bt[0]));
     for (int t = 1; t <= Lmax; ++t) key.push_back(t == Lmax || Bt[t] > Bt[t + 1] ? 1 : 0);  // launches of the small stages
     key.push_back(d_F ? 1 : 0);
     key.push_back(d_sums ? 1 : 0);
