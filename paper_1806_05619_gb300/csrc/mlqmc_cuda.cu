@@ -1404,19 +1404,18 @@ __global__ void __launch_bounds__(256) kb_qoi_part(FmgArgs A, int t, int B, int 
     }
 }
 
-// F_t of samples 0..B-1 from the chunk sums (mean of u, partials added in
-// order) or from the four centre cells (centre QoI).
+// F_t of samples 0..B-1 from the chunk sums (mean of u; a warp per sample, in
+// a fixed order) or from the four centre cells (centre QoI).
 template <typename T, bool U64>
-__global__ void kb_qoi_final(FmgArgs A, int t, int B, int P, const double* __restrict__ part)
+__global__ void __launch_bounds__(256) kb_qoi_final(FmgArgs A, int t, int B, int P, const double* __restrict__ part)
 {
-    const int n = A.lv[t].n;
-    GRID_STRIDE(i, B)
-    {
+    const int n = A.lv[t].n, lane = threadIdx.x & 31;
+    for (int i = blockIdx.x * 8 + (threadIdx.x >> 5); i < B; i += gridDim.x * 8) {
         double v;
         if (A.qoi == MLQMC_QOI_MEAN) {
             double sum = 0.0;
-            for (int q = 0; q < P; ++q) sum += part[static_cast<size_t>(i) * P + q];
-            v = sum / (static_cast<double>(n) * n);
+            for (int q = lane; q < P; q += 32) sum += part[static_cast<size_t>(i) * P + q];
+            v = team_sum(WarpTeam{}, sum, nullptr) / (static_cast<double>(n) * n);
         } else {
             const int m = n / 2;
             const int c[4] = {(m - 1) * n + (m - 1), (m - 1) * n + m, m * n + (m - 1), m * n + m};
@@ -1427,7 +1426,7 @@ __global__ void kb_qoi_final(FmgArgs A, int t, int B, int P, const double* __res
             }
             v = 0.25 * s4;
         }
-        A.F[static_cast<size_t>(i) * A.n_levels + t] = v;
+        if (lane == 0) A.F[static_cast<size_t>(i) * A.n_levels + t] = v;
     }
 }
 
@@ -1715,11 +1714,14 @@ int grid_for(mlqmc_ctx* c, int64_t work, int threads = 256)
     return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(want, static_cast<int64_t>(c->sm_count) * 32)));
 }
 
-// Chunks per sample of the large-level QoI pass (about 65536 cells each).
+// Chunks per sample of the large-level QoI pass, about 4096 cells each: the
+// one CTA that had 65536 cells took 26 us for one 256 x 256 sample and 7 to 14
+// for a small call on 96 x 96 and 128 x 128 (5, and 3.4 to 8 now). The count depends on
+// the level alone, so a sample's F_t has the same bits in any call.
 int qoi_chunks(const mlqmc_ctx* c, int t)
 {
     const int64_t n = c->p.coarse_cells << t;
-    return static_cast<int>(std::max<int64_t>(1, n * n / 65536));
+    return static_cast<int>(std::max<int64_t>(1, n * n / 4096));
 }
 
 // Room for the QoI partial sums of Bt[t] samples on every level t <= Lmax
@@ -2636,8 +2638,8 @@ mlqmc_status fmg_stages(mlqmc_ctx* c, FmgArgs& A, const int* Bt, int Lmax, doubl
                         else kb_qoi_part<T, false, false><<<grid, 256, 0, st>>>(A, t, B, P, c->d_qpart, 1, 0);
                     }
                 }
-                if (refine) kb_qoi_final<T, true><<<grid_for(c, B), 256, 0, st>>>(A, t, B, P, c->d_qpart);
-                else kb_qoi_final<T, false><<<grid_for(c, B), 256, 0, st>>>(A, t, B, P, c->d_qpart);
+                if (refine) kb_qoi_final<T, true><<<grid_for(c, B, 8), 256, 0, st>>>(A, t, B, P, c->d_qpart);
+                else kb_qoi_final<T, false><<<grid_for(c, B, 8), 256, 0, st>>>(A, t, B, P, c->d_qpart);
             }
         }
         if (d_usol) {
@@ -2907,7 +2909,9 @@ mlqmc_status run_chunk(mlqmc_ctx* c, int count, const int* Bt, int Lmax, double*
     if (s != MLQMC_OK) return s;
     if (d_sums) {
         Timed tm(c, kProfReduce, st, work_of<double>(count * (8.0 * p.n_levels + sizeof(SampleDesc)), count * 2.0 * p.n_levels));
-        k_sums<<<p.n_levels * p.n_shifts, 256, 0, st>>>(c->d_samples, count, c->d_F, p.n_levels, p.n_shifts, p.reuse,
+        // a CTA scans all samples: 63 us for the 32,256 of a six-level step with 256 threads, 23 with 1024
+        const int threads = count > 4096 ? 1024 : 256;
+        k_sums<<<p.n_levels * p.n_shifts, threads, 0, st>>>(c->d_samples, count, c->d_F, p.n_levels, p.n_shifts, p.reuse,
                                                         d_sums);
     }
     if (d_Fout) {
