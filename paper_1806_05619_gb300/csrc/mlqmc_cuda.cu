@@ -1497,6 +1497,18 @@ __global__ void k_fout(const SampleDesc* __restrict__ smp, int n, const double* 
 // ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------
+// A round's reuse sums and the device status (cleared) into pinned host memory,
+// out[0] the status bits, out[1..n] the sums: one launch and one wait where the
+// copies to pageable memory and the memset cost several.
+__global__ void __launch_bounds__(256) k_round_out(const double* __restrict__ sums, int n, int* status, double* out)
+{
+    for (int q = threadIdx.x; q < n; q += blockDim.x) out[1 + q] = sums[q];
+    if (threadIdx.x == 0) {
+        *reinterpret_cast<int*>(out) = *status;
+        *status = 0;
+    }
+}
+
 inline bool ok(cudaError_t e) { return e == cudaSuccess; }
 
 size_t align256(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
@@ -2967,6 +2979,7 @@ void free_ctx(mlqmc_ctx* c)
     for (auto& P : c->pools) cudaFree(P.mem);
     if (c->staged) cudaEventDestroy(c->staged);
     cudaFree(c->d_psi_dense);
+    cudaFreeHost(c->h_round);
     cudaFree(c->d_part);
     cudaFree(c->d_qpart);
     cudaFree(c->d_c32);
@@ -2981,7 +2994,6 @@ void free_ctx(mlqmc_ctx* c)
     for (auto e : c->pool) cudaEventDestroy(e);
     if (c->h_samples) cudaFreeHost(c->h_samples);
     if (c->h_count) cudaFreeHost(c->h_count);
-    if (c->h_status) cudaFreeHost(c->h_status);
     delete c;
 }
 
@@ -3191,7 +3203,7 @@ extern "C" mlqmc_status mlqmc_create(const mlqmc_problem* p, int64_t max_samples
            ok(cudaMalloc(&c->d_norms, ms * sizeof(double))) &&
            ok(cudaMalloc(&c->d_active, ms * sizeof(int))) && ok(cudaMalloc(&c->d_count, sizeof(int))) &&
            ok(cudaMallocHost(&c->h_samples, ms * sizeof(SampleDesc))) &&
-           ok(cudaMallocHost(&c->h_count, sizeof(int))) && ok(cudaMallocHost(&c->h_status, sizeof(int))) &&
+           ok(cudaMallocHost(&c->h_count, sizeof(int))) &&
            ok(cudaMalloc(&c->d_status, sizeof(int))) &&
            ok(cudaMalloc(&c->d_queue, sizeof(int))) && ok(cudaMemset(c->d_status, 0, sizeof(int))) &&
            ok(cudaMalloc(&c->d_iters, 2 * MLQMC_MAX_LEVELS * sizeof(int))) &&
@@ -3631,11 +3643,19 @@ namespace mlqmc {
 mlqmc_status fetch_round(mlqmc_ctx* c, const double* d_sums, double* h_sums, size_t n, cudaStream_t st)
 {
     if (!c || (n > 0 && (!d_sums || !h_sums))) return MLQMC_ERR_INVALID_ARG;
-    if ((n > 0 && !ok(cudaMemcpyAsync(h_sums, d_sums, n * sizeof(double), cudaMemcpyDeviceToHost, st))) ||
-        !ok(cudaMemcpyAsync(c->h_status, c->d_status, sizeof(int), cudaMemcpyDeviceToHost, st)) ||
-        !ok(cudaMemsetAsync(c->d_status, 0, sizeof(int), st)) || !ok(cudaStreamSynchronize(st)))
-        return MLQMC_ERR_CUDA;
-    const int h = *c->h_status | c->host_status;
+    if (n + 1 > c->round_cap) {
+        cudaFreeHost(c->h_round);
+        c->h_round = nullptr;
+        c->round_cap = 0;
+        if (!ok(cudaMallocHost(&c->h_round, (n + 1) * sizeof(double)))) return MLQMC_ERR_OOM;
+        c->round_cap = n + 1;
+    }
+    k_round_out<<<1, 256, 0, st>>>(d_sums, static_cast<int>(n), c->d_status, c->h_round);
+    if (last_error() != MLQMC_OK || !ok(cudaStreamSynchronize(st))) return MLQMC_ERR_CUDA;
+    std::memcpy(h_sums, c->h_round + 1, n * sizeof(double));
+    int h = 0;
+    std::memcpy(&h, c->h_round, sizeof(int));
+    h |= c->host_status;
     c->host_status = 0;
     return status_of_bits(h);
 }

@@ -141,6 +141,8 @@ struct mlqmc_ctx {
     double* d_norms = nullptr;
     double* d_part = nullptr;  // partial residual sums of the converged forms (samples x chunks), grown on demand
     int64_t part_cap = 0;
+    double* h_round = nullptr;  // pinned: a round's status and sums (fetch_round)
+    size_t round_cap = 0;
     double* d_qpart = nullptr;  // QoI partial sums of the large levels (samples x chunks), grown on demand
     int64_t qpart_cap = 0;
     // multi-index runs (mlqmc_sample_mixed): per-sample QoI in work order and
@@ -155,7 +157,6 @@ struct mlqmc_ctx {
     int* d_count = nullptr;
     SampleDesc* h_samples = nullptr;  // pinned staging
     int* h_count = nullptr;           // pinned
-    int* h_status = nullptr;          // pinned: the status word read with a round's sums
     cudaEvent_t staged = nullptr;     // recorded after the last copy out of the staging buffer
     // level 0 (its field, faces and banded factorisation) runs on a second
     // stream beside the other levels' fields: fork and join by events; with
