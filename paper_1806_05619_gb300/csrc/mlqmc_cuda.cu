@@ -878,7 +878,8 @@ __global__ void __launch_bounds__(256) kb_rbgs_tile(FmgArgs A, int t, int B, int
 }
 
 // bc of level t-1 = mean over children of (b - A u) on level t.
-// FP64: quad_flux, half the operations of the four children one by one.
+// FP64: quad_flux, half the operations of the four children one by one (two large
+// levels of the six-level step 2.76 -> 1.26 ms).
 template <typename T>
 __global__ void kb_resid_restrict(FmgArgs A, int t, int B, int ones)
 {
@@ -1132,26 +1133,30 @@ __global__ void __launch_bounds__(256) kb_resnorm_part(FmgArgs A, int t, int B, 
     }
 }
 
-// norms[i] = sqrt of the sum of sample i's P partial sums (a warp per sample, in
-// a fixed order: one thread's chain of P dependent FP64 adds took longer than
-// the rest of a small pass), active[i] = (norm_i > thresh); *count = number of
-// active samples.
+// Norm and flag of sample i by one warp: norms[i] = sqrt of the sum of its P
+// partial sums in a fixed order (one thread's chain of P dependent FP64 adds
+// took longer than the rest of a small pass), active[i] = (norm_i > thresh).
+__device__ __forceinline__ int norm_flag(const double* part, int P, double* norms, int* active, int i, double thresh)
+{
+    const int lane = threadIdx.x & 31;
+    double sum = 0.0;
+    for (int q = lane; q < P; q += 32) sum += part[static_cast<size_t>(i) * P + q];
+    sum = team_sum(WarpTeam{}, sum, nullptr);
+    const double nr = sqrt(sum);
+    const int a = nr > thresh ? 1 : 0;
+    if (lane == 0) {
+        norms[i] = nr;
+        active[i] = a;
+    }
+    return a;
+}
+
+// Norms and flags of samples 0..B-1; *count += active samples.
 __global__ void __launch_bounds__(256) kb_norm_flags(const double* part, int P, double* norms, int* active, int B,
                                                      double thresh, int* count)
 {
-    const int lane = threadIdx.x & 31;
-    for (int i = blockIdx.x * 8 + (threadIdx.x >> 5); i < B; i += gridDim.x * 8) {
-        double sum = 0.0;
-        for (int q = lane; q < P; q += 32) sum += part[static_cast<size_t>(i) * P + q];
-        sum = team_sum(WarpTeam{}, sum, nullptr);
-        if (lane == 0) {
-            const double nr = sqrt(sum);
-            norms[i] = nr;
-            const int a = nr > thresh ? 1 : 0;
-            active[i] = a;
-            if (a) atomicAdd(count, 1);
-        }
-    }
+    for (int i = blockIdx.x * 8 + (threadIdx.x >> 5); i < B; i += gridDim.x * 8)
+        if (norm_flag(part, P, norms, active, i, thresh) && (threadIdx.x & 31) == 0) atomicAdd(count, 1);
 }
 
 // Control of a device-side refinement loop (the body of a conditional WHILE
@@ -1159,23 +1164,56 @@ __global__ void __launch_bounds__(256) kb_norm_flags(const double* part, int P, 
 // converged form: at iteration it (iter[0]) with cnt samples above the
 // threshold, stop when cnt = 0; when it has reached max_iter, stop and record
 // NOT_CONVERGED; else run the body once more. iter[MLQMC_MAX_LEVELS] keeps the
-// largest iteration reached. The count is cleared for the next pass.
-__global__ void k_loop_ctl(cudaGraphConditionalHandle h, int* count, int* iter, int max_iter, int* status)
+// largest iteration reached.
+struct LoopCtl {
+    cudaGraphConditionalHandle h;
+    int* iter;  // null: no loop, the host decides
+    int max_iter;
+    int* status;
+};
+
+__device__ __forceinline__ void loop_ctl(const LoopCtl& C, int cnt)
+{
+    const int it = C.iter[0];
+    if (it > C.iter[MLQMC_MAX_LEVELS]) C.iter[MLQMC_MAX_LEVELS] = it;
+    unsigned go = 0;
+    if (cnt > 0) {
+        if (it >= C.max_iter) {
+            atomicOr(C.status, kStatusNotConverged);
+        } else {
+            go = 1;
+            C.iter[0] = it + 1;
+        }
+    }
+    cudaGraphSetConditional(C.h, go);
+}
+
+// The decision from *count, which is cleared for the next pass.
+__global__ void k_loop_ctl(LoopCtl C, int* count)
 {
     const int cnt = *count;
     *count = 0;
-    const int it = iter[0];
-    if (it > iter[MLQMC_MAX_LEVELS]) iter[MLQMC_MAX_LEVELS] = it;
-    unsigned go = 0;
-    if (cnt > 0) {
-        if (it >= max_iter) {
-            atomicOr(status, kStatusNotConverged);
-        } else {
-            go = 1;
-            iter[0] = it + 1;
-        }
-    }
-    cudaGraphSetConditional(h, go);
+    loop_ctl(C, cnt);
+}
+
+// A call of up to kFlagsOne samples (a warp each): norms, flags, their count
+// (into pinned host memory, host loop) or the loop's decision (device loop) in
+// one CTA, in place of a launch with a memset before and a copy or k_loop_ctl
+// after it. With 64 samples one CTA takes 15 us, the two launches 6.
+constexpr int kFlagsOne = 8;
+
+__global__ void __launch_bounds__(256) kb_norm_flags_one(const double* part, int P, double* norms, int* active, int B,
+                                                         double thresh, int* host_count, LoopCtl C)
+{
+    __shared__ int total;
+    if (threadIdx.x == 0) total = 0;
+    __syncthreads();
+    for (int i = threadIdx.x >> 5; i < B; i += 8)
+        if (norm_flag(part, P, norms, active, i, thresh) && (threadIdx.x & 31) == 0) atomicAdd(&total, 1);
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    if (C.iter) loop_ctl(C, total);
+    else *host_count = total;
 }
 
 // Zero n 16-byte words (the correction of a level inside a loop body, where a
@@ -2433,10 +2471,15 @@ mlqmc_status norms_and_ctl(mlqmc_ctx* c, const FmgArgs& A, int t, int B, int P, 
     if (s != MLQMC_OK) return s;
     {
         const int64_t n = c->p.coarse_cells << t;
-        Timed tm(c, kProfReduce, st, work_of<double>(B * (8.0 * P + 12.0), B * 1.0 * P), 2);
-        kb_norm_flags<<<grid_for(c, B, 8), 256, 0, st>>>(c->d_part, P, c->d_norms, c->d_active, B,
-                                                         c->p.refine_rtol * n, c->d_count);
-        k_loop_ctl<<<1, 1, 0, st>>>(h, c->d_count, c->d_iters + t, c->p.refine_max_iter, c->d_status);
+        const LoopCtl ctl{h, c->d_iters + t, c->p.refine_max_iter, c->d_status};
+        const double thresh = c->p.refine_rtol * n;
+        Timed tm(c, kProfReduce, st, work_of<double>(B * (8.0 * P + 12.0), B * 1.0 * P), B <= kFlagsOne ? 1 : 2);
+        if (B <= kFlagsOne) {
+            kb_norm_flags_one<<<1, 256, 0, st>>>(c->d_part, P, c->d_norms, c->d_active, B, thresh, nullptr, ctl);
+        } else {
+            kb_norm_flags<<<grid_for(c, B, 8), 256, 0, st>>>(c->d_part, P, c->d_norms, c->d_active, B, thresh, c->d_count);
+            k_loop_ctl<<<1, 1, 0, st>>>(ctl, c->d_count);
+        }
     }
     return last_error();
 }
@@ -2518,14 +2561,18 @@ mlqmc_status converge_batched(mlqmc_ctx* c, FmgArgs& A, int t, int B, cudaStream
     for (int it = 0;; ++it) {
         const mlqmc_status rs = resnorm<T>(c, A, t, B, P, it > 0 ? c->d_active : nullptr, st);
         if (rs != MLQMC_OK) return rs;
-        if (!ok(cudaMemsetAsync(c->d_count, 0, sizeof(int), st))) return MLQMC_ERR_CUDA;
+        const bool one = B <= kFlagsOne;
+        if (!one && !ok(cudaMemsetAsync(c->d_count, 0, sizeof(int), st))) return MLQMC_ERR_CUDA;
         {
+            const double thresh = c->p.refine_rtol * n;
             Timed tm(c, kProfReduce, st, work_of<double>(B * (8.0 * P + 12.0), B * 1.0 * P));
-            kb_norm_flags<<<grid_for(c, B, 8), 256, 0, st>>>(c->d_part, P, c->d_norms, c->d_active, B,
-                                                             c->p.refine_rtol * n, c->d_count);
+            if (one)
+                kb_norm_flags_one<<<1, 256, 0, st>>>(c->d_part, P, c->d_norms, c->d_active, B, thresh, c->h_count, LoopCtl{});
+            else
+                kb_norm_flags<<<grid_for(c, B, 8), 256, 0, st>>>(c->d_part, P, c->d_norms, c->d_active, B, thresh, c->d_count);
         }
-        if (!ok(cudaMemcpyAsync(c->h_count, c->d_count, sizeof(int), cudaMemcpyDeviceToHost, st)) ||
-            !ok(cudaStreamSynchronize(st)))
+        if ((!one && !ok(cudaMemcpyAsync(c->h_count, c->d_count, sizeof(int), cudaMemcpyDeviceToHost, st))) ||
+            last_error() != MLQMC_OK || !ok(cudaStreamSynchronize(st)))
             return MLQMC_ERR_CUDA;
         c->last_iters[t] = std::max(c->last_iters[t], it);
         if (*c->h_count == 0) break;
@@ -3455,6 +3502,7 @@ mlqmc_status round_graph(mlqmc_ctx* c, int count, const int* Bt, int Lmax, doubl
     for (int t = 0; t <= Lmax; ++t) {
         key.push_back(Bt[t] > 0 ? smoother_for(c, t, Bt[t]) : -1);
         key.push_back(Bt[t] > 0 ? kl_nt_for(c, t, Bt[t]) : 0);
+        key.push_back(Bt[t] <= kFlagsOne ? 1 : 0);
     }
     key.push_back(is_mixed(c->p) ? mlqmc_level0::four_lanes(c->p.coarse_cells, Bt[0]) : level0_lanes(c->p.coarse_cells, Bt[0]));
     for (int t = 1; t <= Lmax; ++t) key.push_back(t == Lmax || Bt[t] > Bt[t + 1] ? 1 : 0);  // launches of the small stages

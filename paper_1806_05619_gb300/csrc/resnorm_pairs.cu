@@ -31,7 +31,7 @@ using namespace mlqmc_dev;
 
 namespace {
 
-constexpr int kCols = 128, kRows = 8, kWarps = 8;  // a warp's strip; a CTA stacks kWarps of them
+constexpr int kCols = 128, kWarps = 8;  // a warp's strip is kCols wide; a CTA stacks kWarps of them
 constexpr uint32_t kAll = 0xffffffffu;
 
 struct Pair {
@@ -107,6 +107,10 @@ __device__ __forceinline__ float4 load_f(const float* p, bool in)
     return in ? *reinterpret_cast<const float4*>(p) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 }
 
+// ROWS: rows of a warp's strip. Eight form the fluxes between strips once in
+// eight rows; two keep the chain of a small level short (one 256 x 256 sample:
+// 13.8 -> 6.2 us).
+template <int ROWS>
 __global__ void __launch_bounds__(32 * kWarps, 2) kb_resnorm_pairs(const __grid_constant__ FmgArgs A, int t, int B,
                                                                    int PX, int P, double* __restrict__ part,
                                                                    const int* __restrict__ active)
@@ -118,8 +122,8 @@ __global__ void __launch_bounds__(32 * kWarps, 2) kb_resnorm_pairs(const __grid_
     for (int w = blockIdx.x; w < B * P; w += gridDim.x) {  // uniform per CTA: every thread reaches block_sum
         const int i = w / P, q = w - i * P;
         if (active && !active[i]) continue;
-        const int x = (q % PX) * kCols + 4 * lane, y0 = ((q / PX) * kWarps + warp) * kRows;
-        const int y1 = min(y0 + kRows, n);
+        const int x = (q % PX) * kCols + 4 * lane, y0 = ((q / PX) * kWarps + warp) * ROWS;
+        const int y1 = min(y0 + ROWS, n);
         const bool in = x < n;                                // x and n multiples of 4: all four cells or none
         const bool east = in && (lane == 31 || x + 4 >= n);   // the strip's last cell owns its east face too
         const double* u = at<double>(A.lv[t].u64, i) + x;
@@ -221,9 +225,10 @@ namespace mlqmc_resnorm {
 bool launch(const FmgArgs& A, int t, int n, int B, double* part, const int* active, int sm_count, cudaStream_t st)
 {
     const int PX = (n + kCols - 1) / kCols, P = chunks(n);
-    static_assert(kRows * kWarps == 64 && kCols == 128, "chunks()");
+    static_assert(kWarps == 8 && kCols == 128, "chunks()");
     const int grid = static_cast<int>(std::min<int64_t>(static_cast<int64_t>(B) * P, static_cast<int64_t>(sm_count) * 16));
-    kb_resnorm_pairs<<<grid, 32 * kWarps, 0, st>>>(A, t, B, PX, P, part, active);
+    if (rows(n) == 2) kb_resnorm_pairs<2><<<grid, 32 * kWarps, 0, st>>>(A, t, B, PX, P, part, active);
+    else kb_resnorm_pairs<8><<<grid, 32 * kWarps, 0, st>>>(A, t, B, PX, P, part, active);
     return cudaGetLastError() == cudaSuccess;
 }
 

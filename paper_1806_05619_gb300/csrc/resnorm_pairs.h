@@ -11,8 +11,11 @@ namespace mlqmc_resnorm {
 // Level sides the kernel takes: rows of whole 16-byte words in every array.
 inline bool supported(int n) { return n % 4 == 0 && n >= 32; }
 
-// Partial sums per sample (tiles of 128 x 64 cells).
-inline int chunks(int n) { return ((n + 127) / 128) * ((n + 63) / 64); }
+// Rows of a warp's strip (by the level alone, so that a sample's norm does not depend on its batch).
+inline int rows(int n) { return n <= 256 ? 2 : 8; }
+
+// Partial sums per sample (tiles of 128 columns and eight strips).
+inline int chunks(int n) { return ((n + 127) / 128) * ((n + 8 * rows(n) - 1) / (8 * rows(n))); }
 
 // bc = 1 - A u64 of level t (n cells per side) for samples 0..B-1 and
 // part[i * chunks(n) + q] = the sum of its squares over tile q. active: null,
