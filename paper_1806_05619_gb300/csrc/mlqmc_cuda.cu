@@ -1764,14 +1764,16 @@ int grid_for(mlqmc_ctx* c, int64_t work, int threads = 256)
     return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(want, static_cast<int64_t>(c->sm_count) * 32)));
 }
 
-// Chunks per sample of the large-level QoI pass, about 4096 cells each: the
-// one CTA that had 65536 cells took 26 us for one 256 x 256 sample and 7 to 14
-// for a small call on 96 x 96 and 128 x 128 (5, and 3.4 to 8 now). The count depends on
-// the level alone, so a sample's F_t has the same bits in any call.
+// Chunks per sample of the large-level QoI pass: about 4096 cells each up to 128
+// cells per side, 8192 up to 256, 32768 above. With one CTA for 65536 cells a
+// 256 x 256 sample took 26 us and a small call on 96 x 96 or 128 x 128 14 and 6.4
+// (7, 8 and 3.4 now); with 4096 everywhere the nine-level step's pass went from
+// 1.20 to 1.5 ms (each chunk ends in an FP64 reduction), so 1.18. The count depends
+// on the level alone, so a sample's F_t has the same bits in any call.
 int qoi_chunks(const mlqmc_ctx* c, int t)
 {
     const int64_t n = c->p.coarse_cells << t;
-    return static_cast<int>(std::max<int64_t>(1, n * n / 4096));
+    return static_cast<int>(std::max<int64_t>(1, n * n / (n <= 128 ? 4096 : n <= 256 ? 8192 : 32768)));
 }
 
 // Room for the QoI partial sums of Bt[t] samples on every level t <= Lmax
