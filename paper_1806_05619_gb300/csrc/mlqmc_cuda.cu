@@ -31,7 +31,7 @@
 #include "rbgs_stream.h"
 #include "rbgs_tma.h"
 #include "resid_tma.h"
-#include "resnorm_pairs.h"
+#include "resnorm_words.h"
 #include "ptx_async.cuh"
 #include "rbgs_whole.h"
 #include "matern_nystrom.h"

@@ -4,83 +4,37 @@
 // In FP64 a cell's residual is nine operations and four widened faces, with
 // r^2 about thirteen slots of a pipe that takes one warp instruction in 64
 // cycles: 1.6 ms for 64 samples of 1024 x 1024, whose 20 bytes per cell move
-// in 0.2 ms. Only the differences u_P - u_Q need FP64 (u64 has all 53 bits, and
-// neighbours cancel to its last ones); a difference is then a pair of FP32
-// numbers to 2^-49 of itself, and fluxes, their sum, the residual and its square
-// are FP32 error-free pairs (as resid_f32x2 does for FP32 iterates). Each
-// difference belongs to a face and is formed once: a warp takes 128 columns,
-// four cells per lane, and walks down eight rows with the fluxes of the row
-// above in registers and the west fluxes of the next lane by shuffles, 2.4 FP64
-// operations per cell in place of thirteen. Four samples x 16 shifts on 1024 x
-// 1024 refined to 1e-10 (the step's 66 such passes on 128 x 128 and above): 45.5
-// -> 29.5 ms for the step, 85 us per pass; one 256 x 256 sample 2.2 -> 2.0 ms,
-// Algorithm 1 on seven levels 4.0 -> 3.4 ms. Now bounded by
-// latency: on 64 samples of 512 x 512 the FP64 pipe is 53 % and the issue slots 45 %
-// busy, DRAM 30 %, with 16 warps of 128 registers per SM.
+// in 0.2 ms. Here only the differences u_P - u_Q are formed in FP64; their
+// products with the faces, the sum over the faces, the scaling and the residual
+// run in three FP32 words per number (flux_words.h), with no more error than the
+// FP64 form: below 2^-62 of the fluxes beyond the differences' own rounding.
+// (Two words left 2^-47 of them: the norm at the FP64 solution rose by a half on
+// 32 x 32 and by a twentieth on 128 x 128, and a tolerance near it was missed.)
+// Four samples x 16 shifts on 1024 x 1024 refined to 1e-10: 45.5 ms for the step
+// with the FP64 form, 29.4 with two words, 30.7 with three.
+// Each difference belongs to a face and is formed once: a warp takes 128
+// columns, four cells per lane, and walks down its rows with the fluxes of the
+// row above in registers and the west fluxes of the next lane by shuffles, 2.4
+// FP64 operations per cell in place of thirteen.
 //
-// Error: a flux k d is off by at most 2^-47 |k d|; d is a difference of
-// neighbours, u/d is at least n/8 for these solutions, so on the levels the
-// kernel takes this stays below what u64's own rounding (2^-53 u) puts into
-// the residual. Values outside FP32's comfortable range (a difference below
-// 2^-74 or beyond 2^127, a residual above 1e15 or not finite) take FP64.
-#include "resnorm_pairs.h"
+// Values outside FP32's comfortable range take other routes: a difference below
+// 2^-74 or from 2^128 on the conversion instructions, a residual above 1e15 or
+// not finite FP64.
+#include "resnorm_words.h"
 
 #include <algorithm>
 #include <cstdint>
 
+#include "flux_words.h"
+
 using namespace mlqmc_dev;
+using mlqmc_words::flux;
+using mlqmc_words::Words;
 
 namespace {
 
 constexpr int kCols = 128, kWarps = 8;  // a warp's strip is kCols wide; a CTA stacks kWarps of them
 constexpr uint32_t kAll = 0xffffffffu;
-
-struct Pair {
-    float h, l;
-};
-
-static __device__ __noinline__ Pair split_rare(double d)
-{
-    Pair p;
-    p.h = __double2float_rn(d);
-    p.l = fabsf(p.h) <= 3.0e38f ? __double2float_rn(d - static_cast<double>(p.h)) : 0.0f;
-    return p;
-}
-
-// d = h + l: the 29 significand bits FP32 has no room for are rounded off h
-// (half up) and make up l, exact but for l's own rounding (2^-49 |d|); bit
-// operations only. Biased exponents 949..1150, where both parts are normal;
-// anything else but zero takes the conversions.
-__device__ __forceinline__ Pair split(double d)
-{
-    const uint32_t hi = static_cast<uint32_t>(__double2hiint(d)), lo = static_cast<uint32_t>(__double2loint(d));
-    const uint32_t e = (hi >> 20) & 0x7FFu;
-    Pair p;
-    if (e - 949u > 201u) {
-        if (((hi << 1) | lo) == 0u) {
-            p.h = p.l = 0.0f;
-            return p;
-        }
-        return split_rare(d);
-    }
-    const uint32_t sgn = hi & 0x80000000u;
-    const uint64_t m = ((static_cast<uint64_t>(hi) << 32) | lo) + 0x10000000ull;
-    const uint32_t mag = __funnelshift_r(static_cast<uint32_t>(m), static_cast<uint32_t>(m >> 32), 29) - 0xC0000000u;
-    p.h = __uint_as_float((mag & 0x7FFFFFFFu) | sgn);
-    const int low = static_cast<int>(static_cast<uint32_t>(m) & 0x1FFFFFFFu) - 0x10000000;
-    p.l = __uint_as_float(__float_as_uint(static_cast<float>(low) * __uint_as_float((e - 948u) << 23)) ^ sgn);
-    return p;
-}
-
-// k (a - b) as a pair.
-__device__ __forceinline__ Pair flux(float k, double a, double b)
-{
-    const Pair d = split(a - b);
-    Pair f;
-    f.h = __fmul_rn(k, d.h);
-    f.l = __fmaf_rn(k, d.l, __fmaf_rn(k, d.h, -f.h));
-    return f;
-}
 
 static __device__ __noinline__ double resid_rare(const FmgArgs* A, int t, int i, int i1, int i2)
 {
@@ -112,7 +66,7 @@ __device__ __forceinline__ float4 load_f(const float* p, bool in)
 // eight rows; two keep the chain of a small level short (one 256 x 256 sample:
 // 13.8 -> 6.2 us).
 template <int ROWS>
-__global__ void __launch_bounds__(32 * kWarps, 2) kb_resnorm_pairs(const __grid_constant__ FmgArgs A, int t, int B,
+__global__ void __launch_bounds__(32 * kWarps, 2) kb_resnorm_words(const __grid_constant__ FmgArgs A, int t, int B,
                                                                    int PX, int P, double* __restrict__ part,
                                                                    const int* __restrict__ active)
 {
@@ -135,7 +89,7 @@ __global__ void __launch_bounds__(32 * kWarps, 2) kb_resnorm_pairs(const __grid_
         double wide = 0.0;
         if (y0 < y1) {
             Row cur, nxt;
-            Pair south[4];  // fluxes of the faces below the row
+            Words south[4];  // fluxes of the faces below the row
             {
                 double below[4];
                 load_u(u + static_cast<ptrdiff_t>(y0 - 1) * n, in && y0 > 0, below);
@@ -166,34 +120,24 @@ __global__ void __launch_bounds__(32 * kWarps, 2) kb_resnorm_pairs(const __grid_
                 nxt.kx = load_f(kx + static_cast<ptrdiff_t>(y + 1) * pitch, in && more);
 
                 const double ul = __shfl_up_sync(kAll, cur.u[3], 1);
-                Pair fx[5];
-                fx[0] = flux(cur.kx.x, cur.u[0], lane == 0 ? uw : ul);
-                fx[1] = flux(cur.kx.y, cur.u[1], cur.u[0]);
-                fx[2] = flux(cur.kx.z, cur.u[2], cur.u[1]);
-                fx[3] = flux(cur.kx.w, cur.u[3], cur.u[2]);
-                fx[4].h = __shfl_down_sync(kAll, fx[0].h, 1);
-                fx[4].l = __shfl_down_sync(kAll, fx[0].l, 1);
-                if (east) fx[4] = flux(ke, ue, cur.u[3]);
-                const float kn[4] = {cur.ky.x, cur.ky.y, cur.ky.z, cur.ky.w};
+                // the fluxes of the cell's west and east faces; the last cell's east one is the next lane's first
+                const Words first = flux(cur.kx.x, cur.u[0], lane == 0 ? uw : ul);
+                Words last;
+                last.h = __shfl_down_sync(kAll, first.h, 1);
+                last.m = __shfl_down_sync(kAll, first.m, 1);
+                last.l = __shfl_down_sync(kAll, first.l, 1);
+                if (east) last = flux(ke, ue, cur.u[3]);
+                const float kn[4] = {cur.ky.x, cur.ky.y, cur.ky.z, cur.ky.w}, ki[3] = {cur.kx.y, cur.kx.z, cur.kx.w};
+                Words west = first;
                 float r[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const Pair north = flux(kn[j], nxt.u[j], cur.u[j]);
-                    // sum of the four outward differences, Sum2
-                    float sh, sl, e;
-                    two_sum32(fx[j].h, -fx[j + 1].h, sh, e);
-                    sl = __fadd_rn(__fsub_rn(fx[j].l, fx[j + 1].l), e);
-                    two_sum32(sh, south[j].h, sh, e);
-                    sl = __fadd_rn(sl, __fadd_rn(e, south[j].l));
-                    two_sum32(sh, -north.h, sh, e);
-                    sl = __fadd_rn(sl, __fsub_rn(e, north.l));
+                    const Words e = j < 3 ? flux(ki[j < 3 ? j : 0], cur.u[j < 3 ? j + 1 : 3], cur.u[j]) : last;
+                    const Words north = flux(kn[j], nxt.u[j], cur.u[j]);
+                    float b, rem;
+                    mlqmc_words::residual(c, west, e, south[j], north, b, rem);
+                    west = e;
                     south[j] = north;
-                    // r = 1 - c s
-                    const float ah = __fmul_rn(c, sh);
-                    const float al = __fmaf_rn(c, sl, __fmaf_rn(c, sh, -ah));
-                    float rh, re, b, rem;
-                    two_sum32(1.0f, -ah, rh, re);
-                    two_sum32(rh, __fsub_rn(re, al), b, rem);
                     if (!(fabsf(b) <= 1.0e15f) && in) {
                         const double v = resid_rare(&A, t, i, x + j, y);
                         b = narrow(v);
@@ -228,8 +172,8 @@ bool launch(const FmgArgs& A, int t, int n, int B, double* part, const int* acti
     const int PX = (n + kCols - 1) / kCols, P = chunks(n);
     static_assert(kWarps == 8 && kCols == 128, "chunks()");
     const int grid = static_cast<int>(std::min<int64_t>(static_cast<int64_t>(B) * P, static_cast<int64_t>(sm_count) * 16));
-    if (rows(n) == 2) kb_resnorm_pairs<2><<<grid, 32 * kWarps, 0, st>>>(A, t, B, PX, P, part, active);
-    else kb_resnorm_pairs<8><<<grid, 32 * kWarps, 0, st>>>(A, t, B, PX, P, part, active);
+    if (rows(n) == 2) kb_resnorm_words<2><<<grid, 32 * kWarps, 0, st>>>(A, t, B, PX, P, part, active);
+    else kb_resnorm_words<8><<<grid, 32 * kWarps, 0, st>>>(A, t, B, PX, P, part, active);
     return cudaGetLastError() == cudaSuccess;
 }
 

@@ -1,5 +1,5 @@
 // Refinement residual with its norm for the converged mixed forms, without the
-// FP64 pipe's sums (resnorm_pairs.cu).
+// FP64 pipe's sums (resnorm_words.cu).
 #pragma once
 
 #include <cuda_runtime.h>
