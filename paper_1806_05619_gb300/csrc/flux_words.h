@@ -15,43 +15,43 @@
 #include <cstring>
 #ifndef __CUDACC__
 #include <cmath>
-#define MLQMC_HD inline
+#define MLQMC_WORDS inline
 #else
-#define MLQMC_HD __host__ __device__ __forceinline__
+#define MLQMC_WORDS __host__ __device__ __forceinline__
 #endif
 
 namespace mlqmc_words {
 
 // One rounding each, never contracted (host code that uses them is compiled with -ffp-contract=off).
 #ifdef __CUDA_ARCH__
-MLQMC_HD float add(float a, float b) { return __fadd_rn(a, b); }
-MLQMC_HD float sub(float a, float b) { return __fsub_rn(a, b); }
-MLQMC_HD float mul(float a, float b) { return __fmul_rn(a, b); }
-MLQMC_HD float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-MLQMC_HD uint32_t hi_word(double d) { return static_cast<uint32_t>(__double2hiint(d)); }
-MLQMC_HD uint32_t lo_word(double d) { return static_cast<uint32_t>(__double2loint(d)); }
-MLQMC_HD float as_float(uint32_t b) { return __uint_as_float(b); }
-MLQMC_HD uint32_t as_bits(float f) { return __float_as_uint(f); }
+MLQMC_WORDS float add(float a, float b) { return __fadd_rn(a, b); }
+MLQMC_WORDS float sub(float a, float b) { return __fsub_rn(a, b); }
+MLQMC_WORDS float mul(float a, float b) { return __fmul_rn(a, b); }
+MLQMC_WORDS float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+MLQMC_WORDS uint32_t hi_word(double d) { return static_cast<uint32_t>(__double2hiint(d)); }
+MLQMC_WORDS uint32_t lo_word(double d) { return static_cast<uint32_t>(__double2loint(d)); }
+MLQMC_WORDS float as_float(uint32_t b) { return __uint_as_float(b); }
+MLQMC_WORDS uint32_t as_bits(float f) { return __float_as_uint(f); }
 #else
-MLQMC_HD float add(float a, float b) { return a + b; }
-MLQMC_HD float sub(float a, float b) { return a - b; }
-MLQMC_HD float mul(float a, float b) { return a * b; }
-MLQMC_HD float fma_rn(float a, float b, float c) { return fmaf(a, b, c); }
-MLQMC_HD uint64_t bits_of(double d)
+MLQMC_WORDS float add(float a, float b) { return a + b; }
+MLQMC_WORDS float sub(float a, float b) { return a - b; }
+MLQMC_WORDS float mul(float a, float b) { return a * b; }
+MLQMC_WORDS float fma_rn(float a, float b, float c) { return fmaf(a, b, c); }
+MLQMC_WORDS uint64_t bits_of(double d)
 {
     uint64_t b;
     memcpy(&b, &d, 8);
     return b;
 }
-MLQMC_HD uint32_t hi_word(double d) { return static_cast<uint32_t>(bits_of(d) >> 32); }
-MLQMC_HD uint32_t lo_word(double d) { return static_cast<uint32_t>(bits_of(d)); }
-MLQMC_HD float as_float(uint32_t b)
+MLQMC_WORDS uint32_t hi_word(double d) { return static_cast<uint32_t>(bits_of(d) >> 32); }
+MLQMC_WORDS uint32_t lo_word(double d) { return static_cast<uint32_t>(bits_of(d)); }
+MLQMC_WORDS float as_float(uint32_t b)
 {
     float f;
     memcpy(&f, &b, 4);
     return f;
 }
-MLQMC_HD uint32_t as_bits(float f)
+MLQMC_WORDS uint32_t as_bits(float f)
 {
     uint32_t b;
     memcpy(&b, &f, 4);
@@ -60,7 +60,7 @@ MLQMC_HD uint32_t as_bits(float f)
 #endif
 
 // a + b = s + e (Knuth)
-MLQMC_HD void two_sum(float a, float b, float& s, float& e)
+MLQMC_WORDS void two_sum(float a, float b, float& s, float& e)
 {
     s = add(a, b);
     const float bb = sub(s, a);
@@ -89,7 +89,7 @@ static Words split_rare(double d)
 // d = h + m + l exactly, for magnitudes from 2^-74 to 2^128 by bit operations:
 // the 29 significand bits below FP32's are rounded off h (half up), as a signed
 // number; its last five are rounded off m in the same way and make up l.
-MLQMC_HD Words split(double d)
+MLQMC_WORDS Words split(double d)
 {
     const uint32_t hi = hi_word(d), lo = lo_word(d);
     const uint32_t e = (hi >> 20) & 0x7FFu;
@@ -112,7 +112,7 @@ MLQMC_HD Words split(double d)
 }
 
 // k (a - b)
-MLQMC_HD Words flux(float k, double a, double b)
+MLQMC_WORDS Words flux(float k, double a, double b)
 {
     const Words d = split(a - b);
     Words f;
@@ -125,7 +125,7 @@ MLQMC_HD Words flux(float k, double a, double b)
 }
 
 // r = 1 - c (west - east + south - north) = b + rem, b rounded to FP32.
-MLQMC_HD void residual(float c, const Words& w, const Words& e, const Words& s, const Words& n, float& b, float& rem)
+MLQMC_WORDS void residual(float c, const Words& w, const Words& e, const Words& s, const Words& n, float& b, float& rem)
 {
     // in pairs, not one after the other: the chains are what a warp waits for
     float h1, h2, h, x1, x2, x3, m1, m2, m3, m4, m5, m, t1, t2, t3, t4, t5, t6;
