@@ -321,6 +321,19 @@ __device__ void synth_level(const TM& tm, const FmgArgs& A, const Lv<T>& L, int 
     tm.sync();
 }
 
+// A product that the compiler may not join with an addition.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
+// hb + sum_j k_j u_j (hb: the rounded product h^2 b), one rounding per face: the
+// sum of a cell's update wherever FP64 sweeps run, so that a sample has the same
+// bits in the kernels of large and of small calls.
+template <typename T>
+__device__ __forceinline__ T gs_sum(T hb, T k0, T u0, T k1, T u1, T k2, T u2, T k3, T u3)
+{
+    return fma(k3, u3, fma(k2, u2, fma(k1, u1, fma(k0, u0, hb))));
+}
+
 // Gauss-Seidel update of one cell: u_P = (h^2 b_P + sum_Q k_PQ u_Q) / D_P.
 // b == null: b = 1; ONES (FP64): known to be (no product: five operations, not six).
 template <typename T, bool ONES>
@@ -329,6 +342,15 @@ __device__ __forceinline__ void gs_cell(const Lv<T>& L, const T* b, T h2, int i1
     const int n = L.n;
     const int p = i2 * n + i1;
     const T* kx = L.kx + i2 * kx_pitch(n);
+    if constexpr (sizeof(T) == 8) {  // gs_sum, without the faces on the boundary
+        T acc = ONES ? h2 : mul_rn(h2, b ? b[p] : T(1));
+        if (i1 > 0) acc = fma(kx[i1], L.u[p - 1], acc);
+        if (i1 < n - 1) acc = fma(kx[i1 + 1], L.u[p + 1], acc);
+        if (i2 > 0) acc = fma(L.ky[i2 * n + i1], L.u[p - n], acc);
+        if (i2 < n - 1) acc = fma(L.ky[(i2 + 1) * n + i1], L.u[p + n], acc);
+        L.u[p] = acc * L.idiag[p];
+        return;
+    }
     T acc = ONES ? h2 : h2 * (b ? b[p] : T(1));
     if (i1 > 0) acc += kx[i1] * L.u[p - 1];
     if (i1 < n - 1) acc += kx[i1 + 1] * L.u[p + 1];
@@ -759,6 +781,38 @@ __device__ double qoi(const TM& tm, const T* u, int n, int kind, double* red)
                              static_cast<double>(u[m * n + (m - 1)]) + static_cast<double>(u[m * n + m]));
     tm.sync();
     return v;
+}
+
+// Sum of the nn <= 4096 cells of a small level of the FP64 form, in one order
+// for the kernels that give a sample a warp (large calls) and those that give it
+// a CTA (small ones): 128 partial sums, of the cells p = c mod 128 in ascending
+// p; then the partial sums c, c + 32, c + 64, c + 96 by sum_of_four, then the 32 by
+// the warp's shuffles.
+__device__ __forceinline__ double sum_of_four(double a, double b, double c, double d) { return (a + c) + (b + d); }
+
+__device__ __forceinline__ double sum128_warp(const double* u, int nn)
+{
+    const int lane = threadIdx.x & 31;
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int p = lane; p < nn; p += 128)
+#pragma unroll
+        for (int w = 0; w < 4; ++w)
+            if (p + 32 * w < nn) s[w] += u[p + 32 * w];
+    return team_sum(WarpTeam{}, sum_of_four(s[0], s[1], s[2], s[3]), nullptr);
+}
+
+// Complete in the first warp; red: 128 values.
+__device__ __forceinline__ double sum128_cta(const double* u, int nn, double* red)
+{
+    const int tid = threadIdx.x;
+    if (tid < 128) {
+        double s = 0.0;
+        for (int p = tid; p < nn; p += 128) s += u[p];
+        red[tid] = s;
+    }
+    __syncthreads();
+    if (tid >= 32) return 0.0;
+    return team_sum(WarpTeam{}, sum_of_four(red[tid], red[tid + 32], red[tid + 64], red[tid + 96]), nullptr);
 }
 
 template <typename T, typename TM>

@@ -7,8 +7,8 @@
 // barrier between phases. The arithmetic of every cell is that of the
 // per-level kernels (kb_rbgs_whole or, on sides it does not take, kb_gs;
 // kb_resid_restrict, kb_prolong, kb_coarse_fixed or kb_coarse,
-// kb_prolong_resid64, kb_resnorm_part): the same bits, except that F_t is
-// summed in another order.
+// kb_prolong_resid64, kb_resnorm_part): the same bits. The FP64 form, which takes
+// these kernels for small calls only, sums F_t in the order of kb_qoi too.
 #pragma once
 
 #include <type_traits>
@@ -25,23 +25,9 @@ using namespace mlqmc_ptx;
 // per-level kernels' sums do: there the compiler joins each sum's first
 // addition with either of its two products (the right-hand side's or the
 // first face's, HEAD; the first or the second face's), kernel by kernel.
-template <typename T>
-__device__ __forceinline__ T mul_rn(T a, T b)
-{
-    if constexpr (sizeof(T) == 4) return __fmul_rn(a, b);
-    else return __dmul_rn(a, b);
-}
-
-// hb + sum_j k_j u_j (hb: the rounded product h^2 b)
-template <typename T>
-__device__ __forceinline__ T gs_sum(T hb, T k0, T u0, T k1, T u1, T k2, T u2, T k3, T u3)
-{
-    return fma(k3, u3, fma(k2, u2, fma(k1, u1, fma(k0, u0, hb))));
-}
-
 // h^2 b + sum_j k_j u_j
 template <typename T, bool HEAD>
-__device__ __forceinline__ T gs_sum(T h2, T b, T k0, T u0, T k1, T u1, T k2, T u2, T k3, T u3)
+__device__ __forceinline__ T gs_sum_b(T h2, T b, T k0, T u0, T k1, T u1, T k2, T u2, T k3, T u3)
 {
     if constexpr (!HEAD) return gs_sum(mul_rn(h2, b), k0, u0, k1, u1, k2, u2, k3, u3);
     return fma(k3, u3, fma(k2, u2, fma(k1, u1, fma(h2, b, mul_rn(k0, u0)))));
@@ -469,7 +455,7 @@ struct Visit {
 #pragma unroll
             for (int x = 0; x < RB; ++x) {
                 if (((x + y) & 1) != COLOUR) continue;
-                const float acc = gs_sum<float, (N > 8)>(h2, b[y][x], kx[y][x], x > 0 ? u[y][x > 0 ? x - 1 : 0] : l, kx[y][x + 1],
+                const float acc = gs_sum_b<float, (N > 8)>(h2, b[y][x], kx[y][x], x > 0 ? u[y][x > 0 ? x - 1 : 0] : l, kx[y][x + 1],
                                       x < RB - 1 ? u[y][x < RB - 1 ? x + 1 : 0] : r, ky[y][x],
                                       y > 0 ? u[y > 0 ? y - 1 : 0][x] : up[x], ky[y + 1][x],
                                       y < RB - 1 ? u[y < RB - 1 ? y + 1 : 0][x] : dn[x]);
@@ -749,7 +735,7 @@ __global__ void __launch_bounds__(256, BIG ? 2 : 3) kb_small_stages(FmgArgs A, P
 {
     static_assert(!CONV || sizeof(T) == 4, "the converged FP64 form keeps its stages level by level");
     extern __shared__ __align__(128) unsigned char smraw[];
-    __shared__ double red[16];
+    __shared__ double red[sizeof(T) == 8 ? 128 : 16];
     uint64_t* bar = reinterpret_cast<uint64_t*>(smraw);
     T* S = reinterpret_cast<T*>(smraw + 128);
     const int i = G.i0 + blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
@@ -766,9 +752,7 @@ __global__ void __launch_bounds__(256, BIG ? 2 : 3) kb_small_stages(FmgArgs A, P
             interpolate<T, NC, false>(C, S + C.oU, su);
             for (int m = 0; m < A.mu0; ++m) vcycle<T, NC, BIG>(P, S, t, A.nu1, A.nu2, false, true);
             if (A.qoi == MLQMC_QOI_MEAN) {
-                double acc = 0.0;
-                for (int p = tid; p < nn; p += nt) acc += su[p];
-                F = mean_of(cta_sum<false>(acc, red));
+                F = mean_of(sum128_cta(su, nn, red));
             } else {
                 const int m = n / 2;
                 F = 0.25 * (su[(m - 1) * n + (m - 1)] + su[(m - 1) * n + m] + su[m * n + (m - 1)] + su[m * n + m]);
@@ -888,7 +872,7 @@ bool attrs(int bytes)
     return good;
 }
 
-constexpr int kMaxSmem = 226 * 1024;
+constexpr int kMaxSmem = 226 * 1024;  // and 1 KB of sums
 
 template <typename T, int NC>
 bool prepare_n0()

@@ -187,8 +187,22 @@ __global__ void k_points_mixed(const SampleDesc* __restrict__ smp, int count, in
 // at fac[(r*(n0+1) + d) * stride + i] (coalesced across samples); the
 // diagonal d = 0 holds 1/L(r, r).
 // ---------------------------------------------------------------------------
+// F_0 of a level-0 solution x(r), r < N: the mean from sixteen partial sums
+// (x of r = c mod 16 in ascending r) added pairwise, or the mean of the four
+// centre cells. One order for the kernels that run a sample on one thread and
+// on several lanes.
+__device__ __forceinline__ double tree16(double (&s)[16])
+{
+#pragma unroll
+    for (int w = 8; w > 0; w >>= 1)
+#pragma unroll
+        for (int c = 0; c < w; ++c) s[c] += s[c + w];
+    return s[0];
+}
+
 // Factor, exact FP64 solve with f = 1, F_0; the mixed forms also keep an FP32
-// copy of the factor for the coarse solves of their FP32 V-cycles.
+// copy of the factor for the coarse solves of their FP32 V-cycles. Every sum
+// takes its oldest term first, as in the kernels on several lanes per sample.
 template <typename T, bool MX>
 __global__ void kb_level0(FmgArgs A, int B)
 {
@@ -203,9 +217,9 @@ __global__ void kb_level0(FmgArgs A, int B)
             const int j1 = j % n0, j2 = j / n0;
             double d = widen(L0.kx[j2 * kx_pitch(n0) + j1]) + widen(L0.kx[j2 * kx_pitch(n0) + j1 + 1]) +
                        widen(L0.ky[j2 * n0 + j1]) + widen(L0.ky[(j2 + 1) * n0 + j1]);
-            for (int q = 1; q <= n0 && q <= j; ++q) {
+            for (int q = n0 < j ? n0 : j; q >= 1; --q) {
                 const double l = fac[static_cast<size_t>(j * W + q) * cs + i];
-                d -= l * l;
+                d = fma(-l, l, d);
             }
             const double rl = rsqrt64(d);
             fac[static_cast<size_t>(j * W) * cs + i] = rl;
@@ -213,7 +227,7 @@ __global__ void kb_level0(FmgArgs A, int B)
                 const int r = j + l;
                 double a = widen(band_a(L0.kx, L0.ky, n0, r, l));
                 for (int tt = (r - n0 > 0 ? r - n0 : 0); tt < j; ++tt)
-                    a -= fac[static_cast<size_t>(r * W + (r - tt)) * cs + i] * fac[static_cast<size_t>(j * W + (j - tt)) * cs + i];
+                    a = fma(-fac[static_cast<size_t>(r * W + (r - tt)) * cs + i], fac[static_cast<size_t>(j * W + (j - tt)) * cs + i], a);
                 fac[static_cast<size_t>(r * W + l) * cs + i] = a * rl;
             }
         }
@@ -222,19 +236,23 @@ __global__ void kb_level0(FmgArgs A, int B)
         const double h2 = 1.0 / (static_cast<double>(n0) * n0);
         for (int r = 0; r < N; ++r) {
             double v = h2;
-            for (int q = 1; q <= n0 && q <= r; ++q) v -= fac[static_cast<size_t>(r * W + q) * cs + i] * x[r - q];
+            for (int q = n0 < r ? n0 : r; q >= 1; --q) v = fma(-fac[static_cast<size_t>(r * W + q) * cs + i], x[r - q], v);
             x[r] = v * fac[static_cast<size_t>(r * W) * cs + i];
         }
         for (int r = N - 1; r >= 0; --r) {
             double v = x[r];
-            for (int q = 1; q <= n0 && r + q < N; ++q) v -= fac[static_cast<size_t>((r + q) * W + q) * cs + i] * x[r + q];
+            for (int q = n0 < N - 1 - r ? n0 : N - 1 - r; q >= 1; --q) v = fma(-fac[static_cast<size_t>((r + q) * W + q) * cs + i], x[r + q], v);
             x[r] = v * fac[static_cast<size_t>(r * W) * cs + i];
         }
         double F0;
         if (A.qoi == MLQMC_QOI_MEAN) {
-            double acc = 0.0;
-            for (int r = 0; r < N; ++r) acc += x[r];
-            F0 = acc / static_cast<double>(N);
+            double acc[16];
+#pragma unroll
+            for (int c = 0; c < 16; ++c) {
+                acc[c] = 0.0;
+                for (int r = c; r < N; r += 16) acc[c] += x[r];
+            }
+            F0 = tree16(acc) / static_cast<double>(N);
         } else {
             const int m = n0 / 2;
             F0 = 0.25 * (x[(m - 1) * n0 + (m - 1)] + x[(m - 1) * n0 + m] + x[m * n0 + (m - 1)] + x[m * n0 + m]);
@@ -269,32 +287,28 @@ __global__ void kb_coarse(FmgArgs A, int B)
         T* xo = at<T>(A.lv[0].u, i);
         T* xs = SM ? reinterpret_cast<T*>(sraw) + threadIdx.x : xo;
         const int xst = SM ? bd : 1;
+        // FP64: oldest term first, as in fmg_small.cuh (FP32: newest first, as there)
         for (int r = 0; r < N; ++r) {
-            T v = h2 * b[r];
-            for (int q = 1; q <= n0 && q <= r; ++q) v -= fac[static_cast<size_t>(r * W + q) * cs + i] * xs[(r - q) * xst];
+            T v = mul_rn(h2, b[r]);
+            const int m = n0 < r ? n0 : r;
+            for (int k = 1; k <= m; ++k) {
+                const int q = sizeof(T) == 8 ? m + 1 - k : k;
+                v = fma(-fac[static_cast<size_t>(r * W + q) * cs + i], xs[(r - q) * xst], v);
+            }
             xs[r * xst] = v * fac[static_cast<size_t>(r * W) * cs + i];
         }
         for (int r = N - 1; r >= 0; --r) {
             T v = xs[r * xst];
-            for (int q = 1; q <= n0 && r + q < N; ++q) v -= fac[static_cast<size_t>((r + q) * W + q) * cs + i] * xs[(r + q) * xst];
+            const int m = n0 < N - 1 - r ? n0 : N - 1 - r;
+            for (int k = 1; k <= m; ++k) {
+                const int q = sizeof(T) == 8 ? m + 1 - k : k;
+                v = fma(-fac[static_cast<size_t>((r + q) * W + q) * cs + i], xs[(r + q) * xst], v);
+            }
             xs[r * xst] = v * fac[static_cast<size_t>(r * W) * cs + i];
         }
         if (SM)
             for (int r = 0; r < N; ++r) xo[r] = xs[r * xst];
     }
-}
-
-// F_0 of a level-0 solution x(r), r < N: the mean from sixteen partial sums
-// (x of r = c mod 16 in ascending r) added pairwise, or the mean of the four
-// centre cells. One order for the kernels that run a sample on one thread and
-// on several lanes.
-__device__ __forceinline__ double tree16(double (&s)[16])
-{
-#pragma unroll
-    for (int w = 8; w > 0; w >>= 1)
-#pragma unroll
-        for (int c = 0; c < w; ++c) s[c] += s[c + w];
-    return s[0];
 }
 
 // Level 0 for n0 = NC fixed at compile time, one thread per sample, with the
@@ -1298,7 +1312,11 @@ __global__ void __launch_bounds__(256) kb_qoi(FmgArgs A, int t, int B, int keep6
                 v = qoi(tm, at<double>(A.lv[t].u64, i), n, A.qoi, red);
             }
         } else {
-            if constexpr (U64) v = qoi(tm, at<double>(A.lv[t].u64, i), A.lv[t].n, A.qoi, red);
+            const int n = A.lv[t].n;
+            if constexpr (U64) v = qoi(tm, at<double>(A.lv[t].u64, i), n, A.qoi, red);
+            else if constexpr (sizeof(T) == 8 && std::is_same<TM, WarpTeam>::value)
+                v = A.qoi == MLQMC_QOI_MEAN ? sum128_warp(at<double>(A.lv[t].u, i), n * n) / (static_cast<double>(n) * n)
+                                            : qoi(tm, at<double>(A.lv[t].u, i), n, A.qoi, red);
             else v = qoi(tm, at<T>(A.lv[t].u, i), A.lv[t].n, A.qoi, red);
         }
         if (tm.leader()) A.F[static_cast<size_t>(i) * A.n_levels + t] = v;

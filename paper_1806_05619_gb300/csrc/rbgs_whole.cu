@@ -164,16 +164,20 @@ __global__ void __launch_bounds__(WGeom<T, N>::TS * WGeom<T, N>::SPC)
             const T w = kr[x], e = kr[x + 1];
             const T nn = sky[c0], so = sky[c0 + N];
             T acc;
-            if constexpr (Gm::F64) {
-                acc = h2;  // b = 1: no product (one FP64 operation in six)
-                if (!ones) acc = h2 * sb[c0];
+            if constexpr (Gm::F64) {  // gs_sum's roundings
+                acc = h2;             // b = 1: no product (one FP64 operation in six)
+                if (!ones) acc = mul_rn(h2, sb[c0]);
             } else {
                 acc = h2 * (ones ? T(1) : sb[c0]);
             }
-            acc += w * (x > 0 ? su[c0 - 1] : T(0));
-            acc += e * (x < N - 1 ? su[c0 + 1] : T(0));
-            acc += nn * (y > 0 ? su[c0 - N] : T(0));
-            acc += so * (y < N - 1 ? su[c0 + N] : T(0));
+            auto face = [&](T k, T v) {
+                if constexpr (Gm::F64) acc = fma(k, v, acc);
+                else acc += k * v;
+            };
+            face(w, x > 0 ? su[c0 - 1] : T(0));
+            face(e, x < N - 1 ? su[c0 + 1] : T(0));
+            face(nn, y > 0 ? su[c0 - N] : T(0));
+            face(so, y < N - 1 ? su[c0 + N] : T(0));
             if constexpr (Gm::F64) su[c0] = acc * sd[c0];  // the stored 1/D, as kb_gs
             else su[c0] = __fdividef(acc, w + e + nn + so);  // hardware reciprocal: within 2 ulp
         }
