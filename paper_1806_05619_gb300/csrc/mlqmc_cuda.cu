@@ -2063,11 +2063,11 @@ mlqmc_status fields_tc(mlqmc_ctx* c, const FmgArgs& A, const int* Bt, int Lmax, 
 // next), above it level 0's factorisation should not wait for the large levels' faces.
 constexpr int64_t kFacesTogether = int64_t{1} << 22;
 
-// Faces of levels 0..Lmax in one launch; false when the call is not of that kind.
-bool faces_together(mlqmc_ctx* c, const FmgArgs& A, const int* Bt, int Lmax, cudaStream_t st)
+// Whether a call forms the faces of its levels in one launch, and their shares of it.
+bool faces_fit(const mlqmc_ctx* c, const int* Bt, int Lmax, FaceLevels& L)
 {
+    L = FaceLevels{};
     if (c->profiling || c->p.coarse_cells % 4 != 0) return false;
-    FaceLevels L{};
     int64_t quads = 0;
     for (int t = 0; t <= Lmax && Bt[t] > 0; ++t) {
         const int64_t n = c->p.coarse_cells << t;
@@ -2076,9 +2076,16 @@ bool faces_together(mlqmc_ctx* c, const FmgArgs& A, const int* Bt, int Lmax, cud
         L.end[t] = static_cast<uint32_t>(quads);
         L.count = t + 1;
     }
-    if (L.count == 0) return false;
+    return L.count > 0;
+}
+
+// Faces of levels 0..Lmax in one launch; false when the call is not of that kind.
+bool faces_together(mlqmc_ctx* c, const FmgArgs& A, const int* Bt, int Lmax, cudaStream_t st)
+{
+    FaceLevels L;
+    if (!faces_fit(c, Bt, Lmax, L)) return false;
     Timed tm(c, kProfSynth, st);
-    kb_faces4_levels<<<grid_for(c, quads), 256, 0, st>>>(A, L);
+    kb_faces4_levels<<<grid_for(c, L.end[L.count - 1]), 256, 0, st>>>(A, L);
     return true;
 }
 
@@ -2324,6 +2331,21 @@ int small_top(const mlqmc_ctx* c, int t_max, Count B)
     return top;
 }
 
+// Largest level whose FMG stages run in one launch per sample (the converged
+// FP64 form keeps its stages level by level); 0: none.
+int stages_top(const mlqmc_ctx* c, const int* Bt, int Lmax)
+{
+    if (!is_mixed(c->p) && c->p.refine_rtol > 0.0) return 0;
+    return small_top(c, Lmax, [Bt](int t) { return Bt[t]; });
+}
+
+// Largest level below t_top whose V-cycle part runs in one launch per sample
+// in a V-cycle on level t_top with B samples; 0: none.
+int vcycle_small_top(const mlqmc_ctx* c, int t_top, int B)
+{
+    return small_top(c, t_top - 1, [B](int) { return B; });
+}
+
 // Algorithmic work of one V-cycle on levels top..0 (faces, right-hand sides
 // and factor in, the top iterate out; the levels' sweeps and transfers).
 template <typename T>
@@ -2426,7 +2448,7 @@ mlqmc_status vcycle_batched(mlqmc_ctx* c, FmgArgs& A, int t_top, int B, bool one
                             bool top_zero = false)
 {
     // the levels below t_top that fit one launch per sample, else the coarse solve alone
-    const int small = small_top(c, t_top - 1, [B](int) { return B; });
+    const int small = vcycle_small_top(c, t_top, B);
     for (int t = t_top; t > small; --t) {
         const int top_ones = (t == t_top && ones) ? 1 : 0;
         // a correction level (and, top_zero, the top level: the first cycle of a
@@ -2629,8 +2651,7 @@ mlqmc_status fmg_stages(mlqmc_ctx* c, FmgArgs& A, const int* Bt, int Lmax, doubl
     // solution output); otherwise, on the TMA interpolation levels, the
     // interpolant itself travels in FP32 (interp32: in the level's field array)
     const int keep64 = (d_usol != nullptr || c->p.qoi != MLQMC_QOI_MEAN) ? 1 : 0;
-    // the small levels' stages in one launch (the converged FP64 form keeps them level by level)
-    const int small = (MX || !refine) ? small_top(c, Lmax, [Bt](int t) { return Bt[t]; }) : 0;
+    const int small = stages_top(c, Bt, Lmax);
     if (small > 0) {
         const mlqmc_status s = small_stages<T>(c, A, Bt, small, d_usol != nullptr, st);
         if (s != MLQMC_OK) return s;
@@ -3516,16 +3537,25 @@ mlqmc_status round_graph(mlqmc_ctx* c, int count, const int* Bt, int Lmax, doubl
     if (!G.body && !ok(cudaStreamCreateWithFlags(&G.body, cudaStreamNonBlocking))) return MLQMC_ERR_CUDA;
     if (!G.in && !ok(cudaEventCreateWithFlags(&G.in, cudaEventDisableTiming))) return MLQMC_ERR_CUDA;
     if (!G.out && !ok(cudaEventCreateWithFlags(&G.out, cudaEventDisableTiming))) return MLQMC_ERR_CUDA;
-    // launch shape: the levels that run and their smoothers, the outputs asked for
+    // launch shape: everything that decides which launches a call consists of
     std::vector<int32_t> key;
+    const int small = stages_top(c, Bt, Lmax);
+    const bool loops = c->p.refine_rtol > 0.0;
+    FaceLevels faces;
     key.push_back(Lmax);
+    key.push_back(small);
+    key.push_back(faces_fit(c, Bt, Lmax, faces) ? 1 : 0);
+    key.push_back(is_mixed(c->p) ? mlqmc_level0::four_lanes(c->p.coarse_cells, Bt[0]) : level0_lanes(c->p.coarse_cells, Bt[0]));
     for (int t = 0; t <= Lmax; ++t) {
         key.push_back(Bt[t] > 0 ? smoother_for(c, t, Bt[t]) : -1);
         key.push_back(Bt[t] > 0 ? kl_nt_for(c, t, Bt[t]) : 0);
-        key.push_back(Bt[t] <= kFlagsOne ? 1 : 0);
+        if (t > small) {
+            key.push_back(vcycle_small_top(c, t, Bt[t]));
+            key.push_back(loops && Bt[t] <= kFlagsOne ? 1 : 0);
+        } else if (t > 0 && t < small) {
+            key.push_back(Bt[t] > Bt[t + 1] ? 1 : 0);  // small_stages launches once per class of finest levels
+        }
     }
-    key.push_back(is_mixed(c->p) ? mlqmc_level0::four_lanes(c->p.coarse_cells, Bt[0]) : level0_lanes(c->p.coarse_cells, Bt[0]));
-    for (int t = 1; t <= Lmax; ++t) key.push_back(t == Lmax || Bt[t] > Bt[t + 1] ? 1 : 0);  // launches of the small stages
     key.push_back(d_F ? 1 : 0);
     key.push_back(d_sums ? 1 : 0);
     // an instantiated graph may still be running the previous call
