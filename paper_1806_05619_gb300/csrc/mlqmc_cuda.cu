@@ -2775,8 +2775,11 @@ void default_smoothers(mlqmc_ctx* c)
 // run, time one V-cycle visit of the level (pre-smoothing and the restricted
 // residual, correction and post-smoothing) of each candidate on 1024 samples
 // of zeroed scratch pools (the timing does not depend on the values) and keep
-// the fastest. Runs once, at creation, on its own stream. The FP64 form takes
-// a fixed rule instead (default_smoothers).
+// the fastest. Runs once, at creation, on its own stream. The scratch stays as
+// the levels' pools, so that the first calls of a small context, and the first
+// rounds of an adaptive run, do not allocate; the levels that run in one launch per
+// sample get theirs too. The FP64 form takes a fixed rule instead
+// (default_smoothers).
 mlqmc_status tune_smoothers(mlqmc_ctx* c)
 {
     default_smoothers(c);
@@ -2791,11 +2794,10 @@ mlqmc_status tune_smoothers(mlqmc_ctx* c)
     mlqmc_status res = MLQMC_OK;
     const int all[4] = {MLQMC_SMOOTHER_GS, MLQMC_SMOOTHER_WHOLE, MLQMC_SMOOTHER_STREAM, MLQMC_SMOOTHER_TMA};
     int large_best[MLQMC_MAX_LEVELS] = {};
-    // the levels that run in one launch per sample need no choice
+    // the levels that run in one launch per sample need no choice, only their pools
     const int fused = small_top(c, c->p.n_levels - 1, [](int) { return 1; });
     for (int t = 1; t < c->p.n_levels && res == MLQMC_OK; ++t)
     for (int cls = 1; cls >= 0 && res == MLQMC_OK; --cls) {  // large batches, then small ones
-        if (t <= fused) continue;
         int cands[4], nc = 0;
         for (int k : all)
             if ((f64 || k != MLQMC_SMOOTHER_GS) && smoother_fits(c, k, t)) cands[nc++] = k;
@@ -2807,6 +2809,7 @@ mlqmc_status tune_smoothers(mlqmc_ctx* c)
             res = MLQMC_ERR_OOM;
             break;
         }
+        if (t <= fused) break;
         for (int u = t - 1; u <= t; ++u) {
             const LevelPool& P = c->pools[u];
             const size_t bytes = level_bytes_per_sample(c->p, c->Ka, u) * static_cast<size_t>(P.cap);

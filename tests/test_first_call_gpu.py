@@ -1,0 +1,25 @@
+"""Mixed forms: the pools of the levels up to 64 cells per side are there after
+creation, so that neither the first call nor the first rounds of Algorithm 1 allocate them."""
+import pytest
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+M = pytest.importorskip("paper_1806_05619_gb300")
+
+
+@pytest.mark.parametrize("n0,levels", [(8, 4), (4, 5)])
+def test_first_call_of_a_small_context_allocates_no_pool(n0, levels):
+    cfg = W.scaled(W.LATTICE_6LEVEL, n0=n0, n_levels=levels, s=24, R=2, precision="mixed_tf32", log2_nmax=12)
+    z, _ = M.cbc_genvec(cfg["s"], cfg["log2_nmax"])
+    sums = torch.zeros(levels * 2 * 2, dtype=torch.float64, device="cuda")
+    warm = M.Context.from_config(cfg, genvec=z)  # the library's own code and tables
+    warm.sample_levels([(levels - 1, 0, 4, 0, 2)], sums)
+    ctx = M.Context.from_config(cfg, genvec=z)
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    ctx.sample_levels([(levels - 1, 0, 512, 0, 2)], sums)  # 1,024 samples: more than 200 MB of pools
+    torch.cuda.synchronize()
+    assert before - torch.cuda.mem_get_info()[0] <= 16 << 20
+    ctx.check_device()
