@@ -3290,7 +3290,8 @@ extern "C" mlqmc_status mlqmc_create(const mlqmc_problem* p, int64_t max_samples
            ok(cudaMalloc(&c->d_Y, ms * p->n_modes * sizeof(double))) &&
            (p->precision == MLQMC_FP64 || ok(cudaMalloc(&c->d_c32, ms * p->n_modes * sizeof(float)))) &&
            ok(cudaMalloc(&c->d_F, ms * p->n_levels * sizeof(double))) &&
-           ok(cudaMalloc(&c->d_chol, ms * c->chol_stride)) && ok(cudaMalloc(&c->d_chol32, ms * c->chol_stride / 2)) &&
+           ((is_mixed(*p) && mlqmc_level0::supported(p->coarse_cells)) || ok(cudaMalloc(&c->d_chol, ms * c->chol_stride))) &&
+           ok(cudaMalloc(&c->d_chol32, ms * c->chol_stride / 2)) &&
            ok(cudaMalloc(&c->d_norms, ms * sizeof(double))) &&
            ok(cudaMalloc(&c->d_active, ms * sizeof(int))) && ok(cudaMalloc(&c->d_count, sizeof(int))) &&
            ok(cudaMallocHost(&c->h_samples, ms * sizeof(SampleDesc))) &&

@@ -136,7 +136,7 @@ struct mlqmc_ctx {
     SampleDesc* d_samples = nullptr;  // rank order (finest level descending)
     double* d_Y = nullptr;            // normals, s per sample
     double* d_F = nullptr;            // F_t per sample, n_levels each
-    double* d_chol = nullptr;         // banded level-0 factor per sample (interleaved by sample)
+    double* d_chol = nullptr;         // banded level-0 factor per sample (interleaved by sample); null where only its FP32 copy is read
     float* d_chol32 = nullptr;        // its FP32 copy (mixed forms)
     double* d_norms = nullptr;
     double* d_part = nullptr;  // partial residual sums of the converged forms (samples x chunks), grown on demand

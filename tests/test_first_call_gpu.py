@@ -1,5 +1,6 @@
-"""Mixed forms: the pools of the levels up to 64 cells per side are there after
-creation, so that neither the first call nor the first rounds of Algorithm 1 allocate them."""
+"""Mixed forms, device memory at creation: the pools of the levels up to 64 cells per
+side are there, so that neither the first call nor the first rounds of Algorithm 1
+allocate them; buffers that nothing reads are not."""
 import pytest
 
 import workloads as W
@@ -23,3 +24,19 @@ def test_first_call_of_a_small_context_allocates_no_pool(n0, levels):
     torch.cuda.synchronize()
     assert before - torch.cuda.mem_get_info()[0] <= 16 << 20
     ctx.check_device()
+
+
+def test_creation_keeps_no_fp64_factor_that_nothing_reads():
+    """Sides whose mixed form factors level 0 in FP32 pairs: of the factors of 65,536
+    samples (8 x 8 cells) only the FP32 one, 151 MB, beside 30 MB of points and sums."""
+    cfg = W.scaled(W.LATTICE_6LEVEL, n0=8, n_levels=1, s=8, R=2, precision="mixed_tf32", log2_nmax=12)
+    z, _ = M.cbc_genvec(cfg["s"], cfg["log2_nmax"])
+    warm = M.Context.from_config(cfg, genvec=z)
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    ctx = M.Context.from_config(cfg, genvec=z)
+    assert before - torch.cuda.mem_get_info()[0] <= 256 << 20
+    sums = torch.zeros(4, dtype=torch.float64, device="cuda")
+    for c in (warm, ctx):
+        c.sample_levels([(0, 0, 64, 0, 2)], sums)
+        c.check_device()
