@@ -1193,7 +1193,9 @@ __global__ void k_loop_ctl(LoopCtl C, int* count)
 // A call of up to kFlagsOne samples (a warp each): norms, flags, their count
 // (into pinned host memory, host loop) or the loop's decision (device loop) in
 // one CTA, in place of a launch with a memset before and a copy or k_loop_ctl
-// after it. With 64 samples one CTA takes 15 us, the two launches 6.
+// after it. With 64 samples one CTA takes 15 us, the two launches 6. Microseconds of
+// a call refined to 1e-10 on 128 x 128, two launches / one: 1 sample 705 / 696, 4: 723 /
+// 711, 8: 836 / 825, 12: 843 / 838, 16: 855 / 852, 24: 871 / 882, 64: 1,029 / 1,094.
 constexpr int kFlagsOne = 8;
 
 __global__ void __launch_bounds__(256) kb_norm_flags_one(const double* part, int P, double* norms, int* active, int B,
@@ -1804,10 +1806,14 @@ mlqmc_status last_error()
 // one thread): 16 samples 47 / 61 / 219, 1,024: 55 / 62 / 251, 2,048: 96 / 63 /
 // 252, 8,192: 358 / 175 / 255, 16,368: 713 / 337 / 281; at n0 = 4 2,048: 19 / 18 / 39,
 // 16,384: 92 / 37 / 43, 32,768: 171 / 73 / 55. The other sides have no
-// thread-per-sample kernel in registers and shared memory (n0 = 6: one lane 159,
-// one thread 181 at 16,384, 306 / 269 at 32,768).
+// thread-per-sample kernel in registers and shared memory. A whole call on level 0
+// with 20 modes, one lane / one thread: n0 = 6, 16,384: 611 / 619, 20,000: 754 / 766,
+// 24,000: 914 / 880, 32,768: 1,228 / 1,144; n0 = 10, 14,400: 1,353 / 1,462, 16,384: 1,551 /
+// 1,527, 20,000: 1,886 / 1,905, 24,000: 2,229 / 2,059, 32,768: 3,032 / 2,338; n0 = 8, 12,000:
+// 618 / 629, 14,400: 701 / 701, 16,384: 843 / 762; n0 = 4 the same within 2 % from
+// 14,400 to 28,000, 32,768: 934 / 898.
 constexpr int kLevel0FourLanes = 1280;
-constexpr int level0_one_thread_from(int n0) { return n0 == 8 ? 13000 : 24000; }
+constexpr int level0_one_thread_from(int n0) { return n0 == 8 ? 13000 : n0 == 4 ? 24000 : 20000; }
 
 // Lanes per window row of the call's level-0 kernel; 0: one thread per sample.
 int level0_lanes(int n0, int B)
@@ -2254,11 +2260,16 @@ mlqmc_status smooth_whole(mlqmc_ctx* c, const FmgArgs& A, int t, int B, int nswe
 // FP64 form: calls with fewer samples on a level than this take its one-launch
 // kernels. FP64 issue bounds the sweeps either way; one launch saves the
 // launches' latency and, past these counts, loses more to its barriers.
-// Microseconds of a call, per level / in one launch: n0 = 8, 32 x 32: 16 samples
-// 499 / 186, 1,024: 895 / 796, 2,048: 1,273 / 1,243, 4,096: 2,122 / 2,332; n0 = 4, 32 x 32: 16:
-// 400 / 187, 256: 445 / 261, 1,024: 670 / 748; n0 = 6, 48 x 48: 1,024: 2,239 / 1,822,
-// 2,048: 3,281 / 3,493.
-constexpr int small_f64_below(int n0) { return n0 == 4 ? 512 : 2048; }
+// Microseconds of a call, per level / in one launch, on the side where the line
+// is tightest: n0 = 4, 64 x 64: 64 samples 694 / 342, 384: 1,029 / 977, 512: 1,181 / 1,280,
+// 1,024: 1,897 / 2,245 (32 x 32: 512: 447 / 427, 1,024: 615 / 675); n0 = 6, 48 x 48:
+// 1,024: 1,996 / 1,644, 1,280: 2,242 / 2,051, 1,536: 2,456 / 2,484, 2,048: 2,925 / 3,178; n0 = 8,
+// 64 x 64: 64: 900 / 367, 1,024: 2,146 / 1,974, 2,048: 3,709 / 3,550, 4,096: 6,637 / 6,772. n0 =
+// 10 has no such line below 4,096 (40 x 40: 4,842 / 3,979; its coarse solve per
+// level keeps the vector in global memory): the others' largest. V-cycles from
+// 128 x 128: n0 = 8, 512: 3,994 / 3,629, 2,048: 12,901 / 12,661; n0 = 4, 256: 2,377 / 2,063, 512:
+// 3,683 / 3,758.
+constexpr int small_f64_below(int n0) { return n0 == 4 ? 512 : n0 == 6 ? 1536 : 2048; }
 
 // Largest level up to t_max whose V-cycle part runs in one launch per sample
 // (fmg_small.cuh) for calls with B(t) samples on level t: the levels up to 64
