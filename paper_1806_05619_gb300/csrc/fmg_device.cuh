@@ -325,14 +325,40 @@ __device__ void synth_level(const TM& tm, const FmgArgs& A, const Lv<T>& L, int 
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 
-// hb + sum_j k_j u_j (hb: the rounded product h^2 b), one rounding per face: the
-// sum of a cell's update wherever FP64 sweeps run, so that a sample has the same
-// bits in the kernels of large and of small calls.
+// The sums of the sweeps and residuals that more than one kernel forms, one
+// rounding per face in an order that is written out, so that a cell has the same
+// bits in the kernels that take a level at a time and in those that keep a
+// sample's levels in one CTA.
+
+// hb + sum_j k_j u_j (hb: the rounded product h^2 b)
 template <typename T>
 __device__ __forceinline__ T gs_sum(T hb, T k0, T u0, T k1, T u1, T k2, T u2, T k3, T u3)
 {
     return fma(k3, u3, fma(k2, u2, fma(k1, u1, fma(k0, u0, hb))));
 }
+
+// h^2 b + sum_j k_j u_j. HEAD: the first product that is rounded by itself is the
+// first face's, else the right-hand side's (FP32 whole-sample sweeps: on sides
+// above 8 the one, on 8 the other).
+template <typename T, bool HEAD>
+__device__ __forceinline__ T gs_sum_b(T h2, T b, T k0, T u0, T k1, T u1, T k2, T u2, T k3, T u3)
+{
+    if constexpr (!HEAD) return gs_sum(mul_rn(h2, b), k0, u0, k1, u1, k2, u2, k3, u3);
+    return fma(k3, u3, fma(k2, u2, fma(k1, u1, fma(h2, b, mul_rn(k0, u0)))));
+}
+
+// sum_j k_j d_j; head: the second face's product is rounded by itself, else the first's
+template <typename T>
+__device__ __forceinline__ T flux_sum(bool head, T k0, T d0, T k1, T d1, T k2, T d2, T k3, T d3)
+{
+    const T a = head ? fma(k0, d0, mul_rn(k1, d1)) : fma(k1, d1, mul_rn(k0, d0));
+    return fma(k3, d3, fma(k2, d2, a));
+}
+
+// Which of the two for child d = (x & 1) + 2 (y & 1) of a coarse cell in the FP32
+// restricted residual: of the whole-sample kernels, and of resid_restrict_cell.
+__device__ __forceinline__ constexpr bool whole_head(int d) { return d != 3; }
+__device__ __forceinline__ constexpr bool cell_head(int d) { return d == 1; }
 
 // Gauss-Seidel update of one cell: u_P = (h^2 b_P + sum_Q k_PQ u_Q) / D_P.
 // b == null: b = 1; ONES (FP64): known to be (no product: five operations, not six).
@@ -342,20 +368,12 @@ __device__ __forceinline__ void gs_cell(const Lv<T>& L, const T* b, T h2, int i1
     const int n = L.n;
     const int p = i2 * n + i1;
     const T* kx = L.kx + i2 * kx_pitch(n);
-    if constexpr (sizeof(T) == 8) {  // gs_sum, without the faces on the boundary
-        T acc = ONES ? h2 : mul_rn(h2, b ? b[p] : T(1));
-        if (i1 > 0) acc = fma(kx[i1], L.u[p - 1], acc);
-        if (i1 < n - 1) acc = fma(kx[i1 + 1], L.u[p + 1], acc);
-        if (i2 > 0) acc = fma(L.ky[i2 * n + i1], L.u[p - n], acc);
-        if (i2 < n - 1) acc = fma(L.ky[(i2 + 1) * n + i1], L.u[p + n], acc);
-        L.u[p] = acc * L.idiag[p];
-        return;
-    }
-    T acc = ONES ? h2 : h2 * (b ? b[p] : T(1));
-    if (i1 > 0) acc += kx[i1] * L.u[p - 1];
-    if (i1 < n - 1) acc += kx[i1 + 1] * L.u[p + 1];
-    if (i2 > 0) acc += L.ky[i2 * n + i1] * L.u[p - n];
-    if (i2 < n - 1) acc += L.ky[(i2 + 1) * n + i1] * L.u[p + n];
+    // gs_sum, without the faces on the boundary
+    T acc = ONES ? h2 : mul_rn(h2, b ? b[p] : T(1));
+    if (i1 > 0) acc = fma(kx[i1], L.u[p - 1], acc);
+    if (i1 < n - 1) acc = fma(kx[i1 + 1], L.u[p + 1], acc);
+    if (i2 > 0) acc = fma(L.ky[i2 * n + i1], L.u[p - n], acc);
+    if (i2 < n - 1) acc = fma(L.ky[(i2 + 1) * n + i1], L.u[p + n], acc);
     L.u[p] = acc * L.idiag[p];
 }
 
@@ -423,7 +441,13 @@ __device__ __forceinline__ T resid_restrict_cell(const Lv<T>& F, const T* b, int
 #pragma unroll
     for (int d = 0; d < 4; ++d) {
         const int i1 = 2 * I1 + (d & 1), i2 = 2 * I2 + (d >> 1);
-        s += (b ? b[i2 * n + i1] : T(1)) - ih2 * apply_h2<T, T>(F.kx, F.ky, F.u, n, i1, i2);
+        const int p = i2 * n + i1;
+        const T* kx = F.kx + i2 * kx_pitch(n) + i1;
+        const T up = F.u[p];
+        const T a2 = flux_sum<T>(cell_head(d), kx[0], up - (i1 > 0 ? F.u[p - 1] : T(0)), kx[1],
+                                 up - (i1 < n - 1 ? F.u[p + 1] : T(0)), F.ky[p], up - (i2 > 0 ? F.u[p - n] : T(0)), F.ky[p + n],
+                                 up - (i2 < n - 1 ? F.u[p + n] : T(0)));
+        s += fma(-ih2, a2, b ? b[p] : T(1));
     }
     return T(0.25) * s;
 }

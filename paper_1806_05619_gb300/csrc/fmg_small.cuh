@@ -21,26 +21,6 @@ namespace {
 using namespace mlqmc_dev;
 using namespace mlqmc_ptx;
 
-// The sums below are written with explicit FMAs, so that they round as the
-// per-level kernels' sums do: there the compiler joins each sum's first
-// addition with either of its two products (the right-hand side's or the
-// first face's, HEAD; the first or the second face's), kernel by kernel.
-// h^2 b + sum_j k_j u_j
-template <typename T, bool HEAD>
-__device__ __forceinline__ T gs_sum_b(T h2, T b, T k0, T u0, T k1, T u1, T k2, T u2, T k3, T u3)
-{
-    if constexpr (!HEAD) return gs_sum(mul_rn(h2, b), k0, u0, k1, u1, k2, u2, k3, u3);
-    return fma(k3, u3, fma(k2, u2, fma(k1, u1, fma(h2, b, mul_rn(k0, u0)))));
-}
-
-// sum_j k_j d_j
-template <typename T>
-__device__ __forceinline__ T flux_sum(bool head, T k0, T d0, T k1, T d1, T k2, T d2, T k3, T d3)
-{
-    const T a = head ? fma(k0, d0, mul_rn(k1, d1)) : fma(k1, d1, mul_rn(k0, d0));
-    return fma(k3, d3, fma(k2, d2, a));
-}
-
 // sides whose per-level smoother is kb_gs and whose coarse solve is kb_coarse
 template <int NC>
 constexpr bool kPlain = NC != 4 && NC != 8;
@@ -109,10 +89,10 @@ __device__ __forceinline__ void restrict_residual(const Level& F, const Level& C
             const int c0 = y * n + x;
             const T up = su[c0];
             const T* kr = skx + y * XP;
-            const T a2 = flux_sum<T>(d == 1, kr[x], up - (x > 0 ? su[c0 - 1] : T(0)), kr[x + 1],
+            const T a2 = flux_sum<T>(cell_head(d), kr[x], up - (x > 0 ? su[c0 - 1] : T(0)), kr[x + 1],
                                      up - (x < n - 1 ? su[c0 + 1] : T(0)), sky[c0], up - (y > 0 ? su[c0 - n] : T(0)),
                                      sky[c0 + n], up - (y < n - 1 ? su[c0 + n] : T(0)));
-            s += (ones ? T(1) : sb[c0]) - ih2 * a2;
+            s += fma(-ih2, a2, ones ? T(1) : sb[c0]);
         }
         S[C.oB + q] = T(0.25) * s;
     }
@@ -507,7 +487,7 @@ __device__ __forceinline__ void visit_down(const Level& L, const Level& C, float
 #pragma unroll
             for (int x = 0; x < RB; ++x) {
                 const float c = v.u[y][x];
-                const float a2 = flux_sum<float>(!((x & 1) && (y & 1)), v.kx[y][x], c - (x > 0 ? v.u[y][x > 0 ? x - 1 : 0] : l),
+                const float a2 = flux_sum<float>(whole_head((x & 1) + 2 * (y & 1)), v.kx[y][x], c - (x > 0 ? v.u[y][x > 0 ? x - 1 : 0] : l),
                                                  v.kx[y][x + 1], c - (x < RB - 1 ? v.u[y][x < RB - 1 ? x + 1 : 0] : rt),
                                                  v.ky[y][x], c - (y > 0 ? v.u[y > 0 ? y - 1 : 0][x] : v.up[x]),
                                                  v.ky[y + 1][x], c - (y < RB - 1 ? v.u[y < RB - 1 ? y + 1 : 0][x] : v.dn[x]));

@@ -164,20 +164,17 @@ __global__ void __launch_bounds__(WGeom<T, N>::TS * WGeom<T, N>::SPC)
             const T w = kr[x], e = kr[x + 1];
             const T nn = sky[c0], so = sky[c0 + N];
             T acc;
-            if constexpr (Gm::F64) {  // gs_sum's roundings
-                acc = h2;             // b = 1: no product (one FP64 operation in six)
+            if constexpr (Gm::F64) {  // gs_sum; b = 1: no product (one FP64 operation in six)
+                acc = h2;
                 if (!ones) acc = mul_rn(h2, sb[c0]);
-            } else {
-                acc = h2 * (ones ? T(1) : sb[c0]);
+                acc = fma(w, x > 0 ? su[c0 - 1] : T(0), acc);
+            } else {  // gs_sum_b<N > 8>
+                const T b = ones ? T(1) : sb[c0], ul = x > 0 ? su[c0 - 1] : T(0);
+                acc = N > 8 ? fma(h2, b, mul_rn(w, ul)) : fma(w, ul, mul_rn(h2, b));
             }
-            auto face = [&](T k, T v) {
-                if constexpr (Gm::F64) acc = fma(k, v, acc);
-                else acc += k * v;
-            };
-            face(w, x > 0 ? su[c0 - 1] : T(0));
-            face(e, x < N - 1 ? su[c0 + 1] : T(0));
-            face(nn, y > 0 ? su[c0 - N] : T(0));
-            face(so, y < N - 1 ? su[c0 + N] : T(0));
+            acc = fma(e, x < N - 1 ? su[c0 + 1] : T(0), acc);
+            acc = fma(nn, y > 0 ? su[c0 - N] : T(0), acc);
+            acc = fma(so, y < N - 1 ? su[c0 + N] : T(0), acc);
             if constexpr (Gm::F64) su[c0] = acc * sd[c0];  // the stored 1/D, as kb_gs
             else su[c0] = __fdividef(acc, w + e + nn + so);  // hardware reciprocal: within 2 ulp
         }
@@ -204,11 +201,10 @@ __global__ void __launch_bounds__(WGeom<T, N>::TS * WGeom<T, N>::SPC)
                 const int c0 = y * N + x;
                 const T up = su[c0];
                 const T* kr = skx + y * XP;
-                T a2 = kr[x] * (up - (x > 0 ? su[c0 - 1] : T(0)));
-                a2 += kr[x + 1] * (up - (x < N - 1 ? su[c0 + 1] : T(0)));
-                a2 += sky[c0] * (up - (y > 0 ? su[c0 - N] : T(0)));
-                a2 += sky[c0 + N] * (up - (y < N - 1 ? su[c0 + N] : T(0)));
-                s += (ones ? T(1) : sb[c0]) - ih2 * a2;
+                const T a2 = flux_sum<T>(whole_head(d), kr[x], up - (x > 0 ? su[c0 - 1] : T(0)), kr[x + 1],
+                                         up - (x < N - 1 ? su[c0 + 1] : T(0)), sky[c0], up - (y > 0 ? su[c0 - N] : T(0)),
+                                         sky[c0 + N], up - (y < N - 1 ? su[c0 + N] : T(0)));
+                s += fma(-ih2, a2, ones ? T(1) : sb[c0]);
             }
             gbc[q] = T(0.25) * s;
         }
