@@ -84,8 +84,9 @@ typedef enum {
  *  precision     mlqmc_precision.
  *  refine_rtol   0: FMG with exactly mu0 V-cycles per level (fixed work).
  *                >0: after the mu0 cycles each level is iterated until
- *                ||b - A u||_2 / ||b||_2 <= refine_rtol (FP64 residual; in the
- *                mixed forms each correction is an FP32 V-cycle solve).
+ *                ||b - A u||_2 / ||b||_2 <= refine_rtol (the residual of the
+ *                FP64 solution to FP64 accuracy; in the mixed forms each
+ *                correction is an FP32 V-cycle solve).
  *  refine_max_iter cap on extra cycles / refinement steps per level.
  *  sampler       mlqmc_sampler.
  *  seed          Philox key: random shifts (lattice) or the normals (MC).
@@ -471,6 +472,13 @@ int64_t mlqmc_launch_count(const mlqmc_ctx* c);
  * 32 x 32 tiles, sides 8, 16 or a multiple of 32; kb_gs's operations in
  * kb_gs's order) but is slower there, FP64 issue being the limit on GB300;
  * the wavefront and TMA smoothers are FP32 only.
+ * Levels up to 64 cells per side of coarsest sides 4, 6, 8 and 10 (FP64: where
+ * they fit in shared memory, for calls of few samples) run in one launch per
+ * sample that holds all of them; its sweeps are those of the smoother that kind
+ * names, in its order (MLQMC_SMOOTHER_WHOLE, or MLQMC_SMOOTHER_TILE / _GS on sides
+ * that are not a power of two). The mixed forms choose and time nothing on these
+ * levels (tuned_ms 0); forcing another smoother on one takes it and the levels
+ * above it out of that launch.
  * mlqmc_set_smoother: force `kind` on `level` (1 <= level < n_levels) for
  * later calls; MLQMC_ERR_INVALID_ARG if that smoother cannot run the level
  * in the context's form (GS in a mixed form, an FP32-only smoother in the
@@ -522,8 +530,8 @@ int64_t mlqmc_graph_replays(const mlqmc_ctx* c);
  * round graphs apply to it (mlqmc_set_round_graphs), it fits one chunk and
  * profiling is off: the descriptors are uploaded by one
  * copy, then the call's kernels are captured into a graph, an instantiated
- * graph of the same launch shape (the levels that run, their smoothers, the
- * outputs asked for) is updated in place (cudaGraphExecUpdate) or a new one
+ * graph of the same launch shape (the levels that run, the kernels that their
+ * sample counts choose, the outputs asked for) is updated in place (cudaGraphExecUpdate) or a new one
  * instantiated, and the graph is launched once. In the converged forms
  * (refine_rtol > 0) each level's refinement loop becomes a conditional WHILE
  * node: its body (the masked mu0 V-cycles, u64 += e, the residual norms and
@@ -550,6 +558,9 @@ mlqmc_status mlqmc_set_round_graphs(mlqmc_ctx* c, int32_t mode);
  * Per-kernel device timing of mlqmc_sample_levels (off by default). With
  * enable = 1 every later launch is bracketed by CUDA events recorded on the
  * launch stream; enable = 0 stops recording. Either call clears the totals.
+ * While it is on, the fields of a call come from one tensor-core launch per
+ * level, so that their time can be told apart (one per tile width otherwise);
+ * the other launches are the same.
  */
 mlqmc_status mlqmc_profile(mlqmc_ctx* c, int32_t enable);
 
@@ -557,8 +568,9 @@ mlqmc_status mlqmc_profile(mlqmc_ctx* c, int32_t enable);
  * Totals since the last mlqmc_profile call, per kernel kind (8 entries):
  * 0 normals, 1 level-0 banded factor and exact solve (per sample), 2 KL field
  * and faces, 3 red-black sweeps, 4 residual/restriction, prolongation and
- * FP64 refinement updates, 5 coarse solves of the V-cycles, 6 QoI, norms,
- * reuse sums and outputs, 7 KL contraction on the tensor cores.
+ * FP64 refinement updates, 5 small levels in one launch per sample (their FMG
+ * stages and their part of the V-cycles, under the finest of them) and coarse
+ * solves of the V-cycles above, 6 QoI, norms, reuse sums and outputs, 7 KL contraction on the tensor cores.
  * out_ms: device milliseconds (host, 8 doubles); out_n: launches (host, 8
  * int64). Waits for the recorded events.
  */

@@ -419,7 +419,8 @@ class Context:
     SMOOTHERS = ["gs", "tile", "stream", "tma", "whole"]
 
     def smoother_info(self):
-        """Per level (smoother name, {name: tuned ms}); level 0 has no sweeps."""
+        """Per level (smoother name, {name: tuned ms}); level 0 has no sweeps, and levels
+        that run in one launch per sample are not timed."""
         kind = (C.c_int32 * self.n_levels)()
         nk = len(self.SMOOTHERS)
         ms = np.zeros(self.n_levels * nk)

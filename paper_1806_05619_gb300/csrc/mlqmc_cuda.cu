@@ -1320,7 +1320,7 @@ __global__ void __launch_bounds__(256) kb_qoi(FmgArgs A, int t, int B, int keep6
 // of sample i with the per-cell work of kb_qoi (UPD: u64 += e, the FP32 copy
 // of u64, the sum; U64 with FP32 work arrays: the FP32 copy and the sum;
 // else the sum) and writes its partial sum; kb_qoi_final adds each sample's
-// partials in order.
+// partials, a warp per sample in a fixed order.
 template <typename T, bool U64, bool UPD>
 __global__ void __launch_bounds__(256) kb_qoi_part(FmgArgs A, int t, int B, int P, double* part, int keep64,
                                                    int interp32)
@@ -2685,7 +2685,7 @@ mlqmc_status fmg_stages(mlqmc_ctx* c, FmgArgs& A, const int* Bt, int Lmax, doubl
                 if (fuse_update) kb_qoi<T, true, WarpTeam, MX><<<grid, 256, 0, st>>>(A, t, B, keep64);
                 else if (refine) kb_qoi<T, true, WarpTeam><<<grid, 256, 0, st>>>(A, t, B, 1);
                 else kb_qoi<T, false, WarpTeam><<<grid, 256, 0, st>>>(A, t, B, 1);
-            } else {  // chunks of a sample over several CTAs, partial sums added in order
+            } else {  // chunks of a sample over several CTAs
                 const int P = qoi_chunks(c, t);
                 const bool pass = fuse_update || (refine && sizeof(T) == 4) || c->p.qoi == MLQMC_QOI_MEAN;
                 const int grid = static_cast<int>(std::min<int64_t>(static_cast<int64_t>(B) * P, c->sm_count * 8));
