@@ -149,7 +149,7 @@ def peaks():
 
 
 KIND_KERNELS = {
-    "points": "k_points", "level0": "kb_level0_fixed", "synth": "kb_synth_G/z, kb_faces",
+    "points": "k_points", "level0": "kb_level0_pairs (mixed), kb_level0_lanes, kb_level0_fixed", "synth": "kb_synth_G/z, kb_faces",
     "transfer": "kb_prolong_resid_tma, kb_resid_restrict, kb_prolong(_resid64)", "coarse": "kb_coarse_fixed",
     "reduce": "kb_qoi(_part), k_sums", "kl_tc": "kl_tc_kernel (tcgen05)",
 }
@@ -160,6 +160,8 @@ SMOOTHER_KERNELS = {"whole": "kb_rbgs_whole", "tma": "kb_rbgs_tma", "stream": "k
 def kernel_name(kind, level, smoothers):
     if kind == "smooth" and level is not None:
         return SMOOTHER_KERNELS[smoothers[level]]
+    if kind == "coarse" and level:  # the small levels of a sample in one launch, under the finest of them
+        return "kb_small_stages, kb_small_vcycle"
     return KIND_KERNELS.get(kind, kind)
 
 
