@@ -4,14 +4,16 @@
 // of samples. Samples are ranked by finest level, descending; every level t
 // keeps a pool with one block of arrays per sample whose FMG reaches t
 // (B_t samples, B_t non-increasing in t), so sample i uses block i at every
-// level. All grid work is level-synchronous: each kb_* kernel is one flat grid
-// over the B_t samples of one level (KL field, faces, red-black sweeps,
-// residual/restriction, prolongation, FP64 refinement steps, QoI), so samples
-// of uneven finest levels share every launch of the levels they have in
-// common (Sec. 4 FMG, Fig. FMG). Only level 0 is per sample: kb_level0 factors
-// the banded level-0 matrix (one warp per sample) and kb_coarse does the
-// coarse solves of the V-cycles (one thread per sample). k_sums then forms the
-// reuse sums (eq. Upsilon-reuse) in a fixed order.
+// level. The grid work of the large levels is level-synchronous: each kb_*
+// kernel is one flat grid over the B_t samples of one level (KL field, faces,
+// red-black sweeps, residual/restriction, prolongation, refinement steps,
+// QoI), so samples of uneven finest levels share every launch of the levels
+// they have in common (Sec. 4 FMG, Fig. FMG). Per sample run the levels up to 64
+// cells per side (fmg_small.cuh: their FMG stages, and their part of the V-cycles
+// above; level by level for coarsest sides other than 4, 6, 8 and 10, forced
+// smoothers and large FP64 calls) and the factor and exact solve of level 0 (lanes
+// or one thread per sample). k_sums then forms the reuse sums (eq. Upsilon-reuse)
+// in a fixed order.
 #include <cuda_runtime.h>
 
 #include <algorithm>
