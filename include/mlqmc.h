@@ -558,9 +558,10 @@ mlqmc_status mlqmc_set_round_graphs(mlqmc_ctx* c, int32_t mode);
  * Per-kernel device timing of mlqmc_sample_levels (off by default). With
  * enable = 1 every later launch is bracketed by CUDA events recorded on the
  * launch stream; enable = 0 stops recording. Either call clears the totals.
- * While it is on, the fields of a call come from one tensor-core launch per
- * level, so that their time can be told apart (one per tile width otherwise);
- * the other launches are the same.
+ * While it is on, the fields and the faces of a call come from one launch per
+ * level each, so that their time can be told apart (otherwise one launch per tile
+ * width forms the fields of all levels, and in small calls that are not replayed
+ * one the faces); the other launches are the same.
  */
 mlqmc_status mlqmc_profile(mlqmc_ctx* c, int32_t enable);
 

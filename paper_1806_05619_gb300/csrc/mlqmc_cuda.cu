@@ -674,35 +674,55 @@ __global__ void kb_faces(FmgArgs A, int t, int B)
 // i2, the east boundary face after the last column and the south boundary
 // faces below the last row. The arithmetic of face_x / face_y, operand for
 // operand.
-__global__ void kb_faces4(FmgArgs A, int t, int B)
+__device__ __forceinline__ void faces4(const FmgArgs& A, int t, uint32_t idx)
 {
     const int n = A.lv[t].n;
     const int q = n >> 2;
     const uint32_t per = static_cast<uint32_t>(n) * static_cast<uint32_t>(q);
-    GRID_STRIDE(idx, B * per)
+    const int i = static_cast<int>(A.lv[t].by_nnq.div(idx));
+    const int p4 = static_cast<int>(idx - i * per);
+    const int i2 = static_cast<int>(A.lv[t].by_nq.div(p4));
+    const int i1 = (p4 - i2 * q) * 4;
+    const float* k = at<float>(A.lv[t].k, i);
+    float* kx = at<float>(A.lv[t].kx, i) + i2 * kx_pitch(n);
+    float* ky = at<float>(A.lv[t].ky, i);
+    const float4 c = *reinterpret_cast<const float4*>(k + i2 * n + i1);
+    const float4 fx = make_float4(i1 > 0 ? hmean(k[i2 * n + i1 - 1], c.x) : 2.0f * c.x, hmean(c.x, c.y),
+                                  hmean(c.y, c.z), hmean(c.z, c.w));
+    *reinterpret_cast<float4*>(kx + i1) = fx;
+    if (i1 + 4 == n) kx[n] = 2.0f * c.w;
+    float4 fy;
+    if (i2 > 0) {
+        const float4 a = *reinterpret_cast<const float4*>(k + (i2 - 1) * n + i1);
+        fy = make_float4(hmean(a.x, c.x), hmean(a.y, c.y), hmean(a.z, c.z), hmean(a.w, c.w));
+    } else {
+        fy = make_float4(2.0f * c.x, 2.0f * c.y, 2.0f * c.z, 2.0f * c.w);
+    }
+    *reinterpret_cast<float4*>(ky + i2 * n + i1) = fy;
+    if (i2 == n - 1)
+        *reinterpret_cast<float4*>(ky + n * n + i1) = make_float4(2.0f * c.x, 2.0f * c.y, 2.0f * c.z, 2.0f * c.w);
+}
+
+__global__ void kb_faces4(FmgArgs A, int t, int B)
+{
+    const int n = A.lv[t].n;
+    GRID_STRIDE(idx, B * (static_cast<uint32_t>(n) * static_cast<uint32_t>(n >> 2))) faces4(A, t, idx);
+}
+
+// The faces of all levels of a small call in one launch: end[l] = quads of the
+// levels up to l (levels below 2^31 quads together).
+struct FaceLevels {
+    uint32_t end[MLQMC_MAX_LEVELS];
+    int count;
+};
+
+__global__ void kb_faces4_levels(FmgArgs A, FaceLevels L)
+{
+    int t = 0;
+    GRID_STRIDE(idx, L.end[L.count - 1])
     {
-        const int i = static_cast<int>(A.lv[t].by_nnq.div(idx));
-        const int p4 = static_cast<int>(idx - i * per);
-        const int i2 = static_cast<int>(A.lv[t].by_nq.div(p4));
-        const int i1 = (p4 - i2 * q) * 4;
-        const float* k = at<float>(A.lv[t].k, i);
-        float* kx = at<float>(A.lv[t].kx, i) + i2 * kx_pitch(n);
-        float* ky = at<float>(A.lv[t].ky, i);
-        const float4 c = *reinterpret_cast<const float4*>(k + i2 * n + i1);
-        const float4 fx = make_float4(i1 > 0 ? hmean(k[i2 * n + i1 - 1], c.x) : 2.0f * c.x, hmean(c.x, c.y),
-                                      hmean(c.y, c.z), hmean(c.z, c.w));
-        *reinterpret_cast<float4*>(kx + i1) = fx;
-        if (i1 + 4 == n) kx[n] = 2.0f * c.w;
-        float4 fy;
-        if (i2 > 0) {
-            const float4 a = *reinterpret_cast<const float4*>(k + (i2 - 1) * n + i1);
-            fy = make_float4(hmean(a.x, c.x), hmean(a.y, c.y), hmean(a.z, c.z), hmean(a.w, c.w));
-        } else {
-            fy = make_float4(2.0f * c.x, 2.0f * c.y, 2.0f * c.z, 2.0f * c.w);
-        }
-        *reinterpret_cast<float4*>(ky + i2 * n + i1) = fy;
-        if (i2 == n - 1)
-            *reinterpret_cast<float4*>(ky + n * n + i1) = make_float4(2.0f * c.x, 2.0f * c.y, 2.0f * c.z, 2.0f * c.w);
+        while (idx >= L.end[t]) ++t;  // idx only grows
+        faces4(A, t, idx - (t > 0 ? L.end[t - 1] : 0u));
     }
 }
 
@@ -1947,12 +1967,12 @@ bool uses_tc(const mlqmc_ctx* c, int t)
     return c->kl_tc && c->d_psi_tc[t] != nullptr;
 }
 
-enum class SynthPart { all, field, faces };
+enum class SynthPart { all, field, faces, idiag };
 
 // Batched KL field and faces of level t for samples 0..B-1. The field comes
 // from the tensor-core contraction (mixed forms, every level)
 // or from the separable SIMT sum; the C operand must already be built.
-// part: the tensor-core field alone, or the faces and 1/D alone (after it).
+// part: the tensor-core field alone, the faces and 1/D alone (after it), or 1/D alone.
 template <typename T>
 mlqmc_status synth_batched(mlqmc_ctx* c, const FmgArgs& A, int t, int B, cudaStream_t st,
                            SynthPart part = SynthPart::all)
@@ -1960,7 +1980,7 @@ mlqmc_status synth_batched(mlqmc_ctx* c, const FmgArgs& A, int t, int B, cudaStr
     LevelTag lt(c, t);
     const int64_t n = c->p.coarse_cells << t;
     if constexpr (sizeof(T) == 4) {
-        if (uses_tc(c, t) && part != SynthPart::faces) {
+        if (uses_tc(c, t) && (part == SynthPart::all || part == SynthPart::field)) {
             const LevelPool& P = c->pools[t];
             float* k = reinterpret_cast<float*>(P.mem + P.off[kK]);
             const double M = static_cast<double>(n * n);
@@ -1974,7 +1994,7 @@ mlqmc_status synth_batched(mlqmc_ctx* c, const FmgArgs& A, int t, int B, cudaStr
                 return MLQMC_ERR_CUDA;
         }
     }
-    if (part == SynthPart::faces) {
+    if (part == SynthPart::faces || part == SynthPart::idiag) {
     } else if (c->matern && (!uses_tc(c, t) || sizeof(T) != 4)) {
         const double M = static_cast<double>(n * n), sm = c->p.n_modes;
         Timed tm(c, kProfSynth, st,
@@ -2006,7 +2026,7 @@ mlqmc_status synth_batched(mlqmc_ctx* c, const FmgArgs& A, int t, int B, cudaStr
     }
     if (part == SynthPart::field) return last_error();
     const double es = sizeof(T), Mc = cells_of(c, t), Fc = faces_of(c, t);
-    {
+    if (part != SynthPart::idiag) {
         Timed tm(c, kProfSynth, st, work_of<T>(B * es * (Mc + 2.0 * Fc), B * 6.0 * Fc));
         if (sizeof(T) == 4 && n % 4 == 0) kb_faces4<<<grid_for(c, B * n * n / 4), 256, 0, st>>>(A, t, B);
         else kb_faces<T><<<grid_for(c, B * n * n), 256, 0, st>>>(A, t, B);
@@ -2044,6 +2064,43 @@ mlqmc_status fields_tc(mlqmc_ctx* c, const FmgArgs& A, const int* Bt, int Lmax, 
         if (!mlqmc_kl::launch(c->kl_variant, f, count, c->p.n_modes, c->d_status, st, nt)) return MLQMC_ERR_CUDA;
     }
     return MLQMC_OK;
+}
+
+// Cells of a call's levels together up to which one launch forms all faces, in
+// calls that are enqueued or captured for one launch (adaptive rounds): a launch
+// per level costs host time there. Per level / in one launch, means of four pairs
+// of runs: Algorithm 1 on nine levels 2,428 / 2,406 us, on seven levels, refined,
+// 3,428 / 3,410. The launch stands before the fork, so the level-0 factorisation
+// waits for every level's faces: a replayed graph, which has no such host time, takes
+// 175 / 178 us for the first round on 128 x 128 and 1 to 5 % more between 2^18 and 2^22
+// cells, and enqueued calls from 2^20 cells 1 to 5 % more.
+constexpr int64_t kFacesTogether = int64_t{1} << 18;
+
+// Whether a call forms the faces of its levels in one launch, and their shares
+// of it (not while a repeated call is captured for replay).
+bool faces_fit(const mlqmc_ctx* c, const int* Bt, int Lmax, FaceLevels& L)
+{
+    L = FaceLevels{};
+    if (c->profiling || c->p.coarse_cells % 4 != 0 || (c->graph.capturing && !c->graph.round_capture)) return false;
+    int64_t quads = 0;
+    for (int t = 0; t <= Lmax && Bt[t] > 0; ++t) {
+        const int64_t n = c->p.coarse_cells << t;
+        quads += Bt[t] * n * (n / 4);
+        if (4 * quads > kFacesTogether) return false;
+        L.end[t] = static_cast<uint32_t>(quads);
+        L.count = t + 1;
+    }
+    return L.count > 0;
+}
+
+// Faces of levels 0..Lmax in one launch; false when the call is not of that kind.
+bool faces_together(mlqmc_ctx* c, const FmgArgs& A, const int* Bt, int Lmax, cudaStream_t st)
+{
+    FaceLevels L;
+    if (!faces_fit(c, Bt, Lmax, L)) return false;
+    Timed tm(c, kProfSynth, st);
+    kb_faces4_levels<<<grid_for(c, L.end[L.count - 1]), 256, 0, st>>>(A, L);
+    return true;
 }
 
 // C operand of the tensor-core contraction for samples 0..count-1 (normals in rank order).
@@ -2940,18 +2997,19 @@ mlqmc_status run_chunk(mlqmc_ctx* c, int count, const int* Bt, int Lmax, double*
         // the persistent contractions cannot start beside the factorisation's
         // CTAs (both need most of an SM's shared memory): the main stream
         // forms every level's field first, level 0's faces and factorisation
-        // follow on the side stream, beside the other levels' faces (all
-        // levels' faces in one launch before the fork, tried for small calls,
-        // hold up the factorisation: a replayed first round of an adaptive run on
-        // 128 x 128 178 us against 175)
+        // follow on the side stream, beside the other levels' faces
+        // (a small call that is not captured for replay: all levels' faces in one
+        // launch before the fork)
         s = fields_tc(c, A, Bt, Lmax, st);
+        const bool together = s == MLQMC_OK && faces_together(c, A, Bt, Lmax, st);
+        const SynthPart rest = together ? SynthPart::idiag : SynthPart::faces;
         if (!ok(cudaEventRecord(c->ev_fields, st)) || !ok(cudaStreamWaitEvent(c->side, c->ev_fields, 0)))
             s = MLQMC_ERR_CUDA;
-        if (s == MLQMC_OK) s = synth_batched<float>(c, A, 0, Bt[0], c->side, SynthPart::faces);
+        if (s == MLQMC_OK) s = synth_batched<float>(c, A, 0, Bt[0], c->side, rest);
         if (s == MLQMC_OK) s = launch_level0(c, A, Bt[0], c->side);
         if (!ok(cudaEventRecord(c->ev_join, c->side))) s = MLQMC_ERR_CUDA;
         for (int t = 1; s == MLQMC_OK && t <= Lmax && Bt[t] > 0; ++t)
-            s = synth_batched<float>(c, A, t, Bt[t], st, SynthPart::faces);
+            s = synth_batched<float>(c, A, t, Bt[t], st, rest);
     } else {
         s = is_mixed(p) ? synth_batched<float>(c, A, 0, Bt[0], c->side) : synth_batched<double>(c, A, 0, Bt[0], c->side);
         if (s == MLQMC_OK) s = launch_level0(c, A, Bt[0], c->side);
@@ -3507,8 +3565,10 @@ mlqmc_status round_graph(mlqmc_ctx* c, int count, const int* Bt, int Lmax, doubl
     std::vector<int32_t> key;
     const int small = stages_top(c, Bt, Lmax);
     const bool loops = c->p.refine_rtol > 0.0;
+    FaceLevels faces;
     key.push_back(Lmax);
     key.push_back(small);
+    key.push_back(faces_fit(c, Bt, Lmax, faces) ? 1 : 0);
     key.push_back(is_mixed(c->p) ? mlqmc_level0::four_lanes(c->p.coarse_cells, Bt[0]) : level0_lanes(c->p.coarse_cells, Bt[0]));
     for (int t = 0; t <= Lmax; ++t) {
         key.push_back(Bt[t] > 0 ? smoother_for(c, t, Bt[t]) : -1);
