@@ -237,6 +237,8 @@ struct mlqmc_ctx {
         std::vector<RoundExec> round_execs;
         int64_t round_launches = 0, round_updates = 0, round_instantiations = 0;
     } graph;
+    std::vector<unsigned char*> retired;  // old blocks of grown pools (kRetiredBytes together at most)
+    size_t retired_bytes = 0;
     uint64_t pool_epoch = 0;  // bumped whenever a pool or device buffer is reallocated
 
     int* d_status = nullptr;  // deferred device status bits
